@@ -716,8 +716,9 @@ __global__ void __launch_bounds__(TX * TY, (TX * TY >= 256 ? 2 : 4))
 
         if (DIM == 3) {
             // planes j = 0 .. 2R-1 (z0-R .. z0+R-1) give the face z0 - 1/2;
-            // phase P of z0 needs up to j = 2R (MUSCL)
-            wait_planes(seq_base + (MUSCL ? 2 * R : 2 * R - 1));
+            // phase P (MUSCL) or phase F (first order: the column value of z0 + 1)
+            // of z0 needs plane j = 2R too
+            wait_planes(seq_base + 2 * R);
             __syncthreads();
             if (flags[0]) { aborted = true; break; }
             if (!MUSCL) {

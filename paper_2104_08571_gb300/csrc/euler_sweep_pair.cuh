@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(256, PairCfg<DIM, LAYOUT, SCHEME>::MIN_CTAS)
         producer_step(seq_base);
 
         if (DIM == 3) {
-            wait_planes(seq_base + (MUSCL ? 2 * R : 2 * R - 1));
+            wait_planes(seq_base + 2 * R);
             __syncthreads();
             if (flags[0]) { aborted = true; break; }
             if (pthr) {

@@ -104,6 +104,18 @@ def test_force_split_fp32_3d_walks(ctx, layout, bc):
     assert_parity(got, tiled.astype(np.float64), 1e-6, 1e-5)
 
 
+@pytest.mark.parametrize("layout", [R.RIPPLE_SOA, R.RIPPLE_AOS])
+def test_force_split_fp64_3d_many_items_per_cta(ctx, layout):
+    """More work items than resident CTAs: the first plane of a CTA's second
+    item has to wait for the plane above it, which the TMA ring is still loading."""
+    dims = (101, 93, 93)
+    U0 = _random_state(dims, seed=17, amp=0.3)
+    ref, _ = oracle.euler_run(U0, 2, scheme=oracle.FORCE_SPLIT)
+    for _ in range(3):
+        got, _ = gpu_euler(ctx, U0, 2, layout=layout, scheme=FORCE)
+        assert_parity(got, ref, 1e-12, LINF_F64)
+
+
 @pytest.mark.parametrize("ndim,dims", [(2, (40, 21)), (3, (18, 9, 12))])
 @pytest.mark.parametrize("dtype", [R.RIPPLE_F64, R.RIPPLE_F32])
 def test_force_split_uniform_state_bit_exact(ctx, ndim, dims, dtype):
