@@ -634,19 +634,46 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
                        : p->scheme == RIPPLE_FORCE_SPLIT    ? SCHEME_FORCE
                                                             : SCHEME_RUSANOV1;
     const bool split = scheme == SCHEME_FORCE;
-    int v = U->variant;
+    // Planes per z work item of variant c: items run in rounds of the resident
+    // CTAs, each costing its planes plus about one (pipeline fill, the z states
+    // below its first plane), so the chunk with the fewest plane times over all
+    // rounds, up to 16 planes: longer ones spread the planes in flight over
+    // more of the field and lose L2 hits (256^3: 16 planes 499 us a step, 33 536,
+    // 66 568).  A fixed 32 left most SMs idle on small grids (48^3
+    // MUSCL-Hancock: 8 items on 152 SMs, 146 us a step; 2 planes per item 15 us).
+    auto z_split = [&](int c, int* chunk) -> double {
+        const long long tiles = (long long)((g.n[0] + kSweepVariants[c].tx - 1) / kSweepVariants[c].tx) *
+                                ((g.n[1] + kSweepVariants[c].ty - 1) / kSweepVariants[c].ty);
+        const long long slots = (long long)std::max(1, sweep_occ(U->dtype, U->ndim, layout, scheme, c)) * ctx->sm_count;
+        double best = 1e300;
+        *chunk = 1;
+        for (int zc = std::min(g.n[2], 16); zc >= 1; --zc) {
+            const long long items = tiles * ((g.n[2] + zc - 1) / zc);
+            const double cost = (double)((items + slots - 1) / slots) * (zc + 1.0);
+            if (cost < best) {
+                best = cost;
+                *chunk = zc;
+            }
+        }
+        return best;
+    };
+    int v = U->variant, zc = U->zchunk;
     if (v < 0 || sweep_smem(U->dtype, U->ndim, layout, scheme, v) == 0) {
-        // default: the row kernel where it exists (FP32 3D MUSCL-Hancock) for SoA
-        // fields, else the packed pair kernel (FP32), else the first that fits.
-        // (AoS planes staged in shared memory put a row's cells 20 bytes apart,
-        // so the row kernel's per-lane loads of an AoS plane conflict in the
-        // shared-memory banks: measured 0.71 against 0.60 ms per 256^3 step for
-        // the pair kernel, whose items read AoS planes in a friendlier order.)
-        const bool row_ok = layout == LAYOUT_SOA && sweep_smem(U->dtype, U->ndim, layout, scheme, kRowVariant) > 0;
-        v = row_ok ? kRowVariant : sweep_smem(U->dtype, U->ndim, layout, scheme, kPairVariant) > 0 ? kPairVariant : -1;
+        // default: the packed pair kernel (FP32), else the first that fits
+        v = sweep_smem(U->dtype, U->ndim, layout, scheme, kPairVariant) > 0 ? kPairVariant : -1;
         for (int c = 0; c < kNumSweepVariants && v < 0; ++c)
             if (sweep_smem(U->dtype, U->ndim, layout, scheme, c) > 0) v = c;
         if (v < 0) return fail(RIPPLE_ERR_INTERNAL, "no sweep kernel fits this configuration");
+        // FP32 3D MUSCL-Hancock SoA fields: the row kernel where its wide tiles fill
+        // the rounds (a plane of its 64 x 14 tile takes 3.8 us with one CTA per
+        // SM, one of the pair kernel's 32 x 8 tile 2.3 us with two): 256^3 500
+        // against 545 us a step, 150 x 101 x 131 106 against 95 us.  (AoS planes
+        // staged in shared memory put a row's cells 20 bytes apart, so the row
+        // kernel's loads of them conflict: 633 against 601 us at 256^3.)
+        if (layout == LAYOUT_SOA && sweep_smem(U->dtype, U->ndim, layout, scheme, kRowVariant) > 0) {
+            int zr, zp;
+            if (3.8 * z_split(kRowVariant, &zr) < 2.3 * z_split(kPairVariant, &zp)) v = kRowVariant;
+        }
         // a 2D grid with fewer tiles than SMs: the shorter tile spreads it over more SMs
         // (the one-cell-per-item 32x4 variant; FP64 arithmetic is the bound there)
         auto tiles = [&](int c) {
@@ -657,6 +684,7 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
             sweep_smem(U->dtype, U->ndim, layout, scheme, 1) > 0 && tiles(1) > tiles(v))
             v = 1;
     }
+    if (U->ndim == 3 && zc <= 0) z_split(v, &zc);
     const int tx = kSweepVariants[v].tx, ty = kSweepVariants[v].ty;
     const double inv_dx[3] = {1.0 / p->dx[0], 1.0 / p->dx[1], U->ndim == 3 ? 1.0 / p->dx[2] : 0.0};
 
@@ -680,7 +708,6 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     L.sg.tiles_x = (g.n[0] + tx - 1) / tx;
     L.sg.tiles_y = (g.n[1] + ty - 1) / ty;
     if (U->ndim == 3) {
-        int zc = U->zchunk > 0 ? U->zchunk : 32;
         zc = std::min(zc, g.n[2]);
         L.sg.zchunk = zc;
         L.sg.chunks_z = (g.n[2] + zc - 1) / zc;

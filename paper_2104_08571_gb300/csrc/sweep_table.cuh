@@ -78,11 +78,14 @@ struct SweepEntry {
         if constexpr (!fits) {
             return 0;
         } else {
-            auto k = K::fn();
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
-                return 0;
-            int n = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, C::NT, C::SMEM) != cudaSuccess) return 0;
+            static const int n = [] {  // the same on every device the library is built for
+                auto k = K::fn();
+                int c = 0;
+                if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess ||
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k, C::NT, C::SMEM) != cudaSuccess)
+                    return 0;
+                return c;
+            }();
             return n;
         }
     }
