@@ -1,436 +1,291 @@
-// FP32 2D and 3D sweeps of the dimensionally split FORCE step (the paper's
+// FP32 2D and 3D steps of the dimensionally split FORCE solver (the paper's
 // own Euler solver, Section 7.3, Listing euler_graph) on strip walks, sm_103a.
 //
-// One sweep of the split step reads the one-cell neighbours along a single
-// axis, so it needs no tile and no block barrier.  Each warp walks a strip
-// 64 cells wide along the swept axis, one chunk of 64 cells (one row
-// segment) at a time; every lane owns a pair of x-adjacent cells held as
-// f32x2 values, so the flux and update arithmetic issues once for two cells
-// (pair_math.cuh).
-//   x sweep (AXIS 0): a walk runs along a row (one y, one z).  Lane l
-//     evaluates the right faces of its two cells as one pair; the left faces
-//     are lane l - 1's right faces (a shuffle) and, for lane 0, the last face
-//     of the previous chunk, carried in registers.  The right neighbour of
-//     lane 31 is the first cell after the chunk, staged with it.
-//   y or z sweep (AXIS 1, 2): a walk runs along the swept axis through the
-//     rows of a 64-column strip (of one z plane for y, one y row for z); the
-//     face below a row is the face above the next one.  The two differ only
-//     in the stride between rows.
-// Either way every face of a walk is evaluated once; the first face of a walk
-// is evaluated again by the walk before it (the host makes walks long enough
-// that this stays a few per cent of the arithmetic).
+// One step is x, then y (then z) sweeps, each a flux difference along one
+// axis of the state the sweep before it left.  The x and y sweeps are fused: a
+// warp walks a strip of columns along y; each new row is swept along x in
+// registers (neighbours and left faces by shuffles) and at once enters the y
+// sweep as the upper row of a face, so the x-swept state never leaves the
+// registers.  In 3D the walk stays in one z plane and writes the x- and
+// y-swept state to the other buffer, and walks along z in a second phase of
+// the same launch bring it back.  HBM traffic per cell update: 32 B in 2D (one
+// sweep per launch moved 64 B), 80 B in 3D (120 B).
 //
-// Staging: every warp owns a ring of NS shared-memory slots of one chunk
-// (1 KB) each, filled by per-thread asynchronous copies (cp.async) NS - 1
-// chunks (x) or NS - 2 rows (y) ahead of the arithmetic, so the loads in
-// flight cost no registers.  A thread waits for its own copy groups only
-// (cp.async.wait_group), so no wait can hang, and no CTA barrier is needed.
-// AoS lanes copy exactly the cells they read (two 16-byte cells); SoA chunks
-// move as 16-byte copies that span two lanes' pairs (half the copies of
-// per-lane 8-byte ones, measured 2 % faster), so there __syncwarp publishes
-// the lanes' copies to each other and ends their reads of a slot before it
-// is refilled (AoS without the barrier: 1 % faster).  Stores are
-// coalesced and direct.  dt, t and the CFL maximum follow the tiled sweep: dt
-// from the wave-speed maximum of the step's input state; the last sweep of a
-// step advances t and reduces the maximum of the new state.  Cells on the
-// boundary write their ghost images for the next sweep, as in every sweep.
+// Lanes: 64 columns x0 - 2 .. x0 + 61 of which the walk updates the 60 columns
+// x0 .. x0 + 59; the two pairs at the ends only supply the x faces.  The pair
+// width keeps every access of an aligned 8 bytes, and 60 of 64 costs less
+// than a separate evaluation of the edge faces of every row.
+// Rows: a walk updates rows y0 .. y1 - 1 and sweeps rows y0 - 1 .. y1 along x
+// (two rows twice per segment).  A row outside the field is the interior row
+// its ghost row would copy (walk_map): its x sweep gives the ghost row of the
+// x-swept state, which is what refilling the padding between the sweeps gives.
+// Faces shared by two walks are evaluated by both from the same values in the
+// same order, so they have the same bits and the step stays conservative.
+//
+// The face: with a, b its states, F_a, F_b their physical fluxes (formed once
+// per cell and handed to the neighbour), the flux of the Richtmyer state
+//   q = (a + b)/2 - (dt/dx)/2 (F_b - F_a)
+// is evaluated at 2q (the flux is homogeneous of degree one), and
+//   V = F_a + F_b + F(2q) - (dx/dt)(b - a)
+// is four times the FORCE flux; the factor goes into the update's dt/dx.
+// Packed pair arithmetic throughout (pair_math.cuh).
+//
+// Staging: each lane copies its own pair of the coming rows into its part of
+// a per-warp ring of kForceSlots slots with cp.async, so loads in flight hold
+// no registers and no wait involves another thread.
+//
+// Measured (SoA, per step, one sweep per launch before -> now): 4096^2 250 ->
+// 117 us, 256^3 630 -> 302 us, 200 x 171 x 186 300 -> 135 us, 64^3 19 us.
+// Bound by issue: 280 warp instructions per 64-column row in 2D, 117 of them
+// packed arithmetic, at 52 % issue; HBM would allow 80 us at 4096^2.
 #pragma once
-#include <cstdint>
-
-#include "euler_sweep.cuh"
-#include "pair_math.cuh"
+#include "walk_common.cuh"
 
 namespace ripple {
 
-template <int DIM, int NS_>
-struct WalkCfg {
-    static constexpr int NC = DIM + 2;
-    static constexpr int NS = NS_;                                // ring slots per warp
-    static constexpr int SLOT = ((64 * NC + NC + 3) / 4) * 4;     // floats: a chunk + lane 31's right neighbour
-    static constexpr int SMEM = kWalkWarps * NS * SLOT * 4;       // dynamic shared memory per CTA
-    static_assert(NS >= 3, "the y and z sweeps keep two rows resident");
-};
-constexpr int kWalkSlots = 6;
+constexpr int kForceSlots = 4;   // ring slots (rows) per warp
+template <int DIM>
+constexpr int force_smem() { return kWalkWarps * kForceSlots * 64 * (DIM + 2) * 4; }
 
-template <int DIM, int LAYOUT, int AXIS, int NS>
-__global__ void __launch_bounds__(kWalkWarps * 32, 2)
-    euler_force_walk_kernel(const float* __restrict__ in, float* __restrict__ out, FieldCtl* __restrict__ ctl,
-                            const WalkGeom wg, const SweepParams prm)
+// Four times the FORCE flux along D of the faces between a and b.
+template <int DIM, int D>
+__device__ __forceinline__ void force4(const f2 (&a)[DIM + 2], const f2 (&b)[DIM + 2], const f2 (&Fa)[DIM + 2],
+                                       const f2 (&Fb)[DIM + 2], f2 gm1, f2 ndtdx, f2 ndxdt, f2 (&V)[DIM + 2])
 {
-    constexpr int NC = DIM + 2, SLOT = WalkCfg<DIM, NS>::SLOT;
-    // 2D AoS cells are 16 bytes: a lane stages exactly the two cells it reads.
-    // Otherwise a chunk moves as 16-byte pieces that span several lanes' cells,
-    // published to the warp by __syncwarp.
-    constexpr bool kOwnCells = LAYOUT == LAYOUT_AOS && NC == 4;
-    const FieldGeom& g = wg.f;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    extern __shared__ __align__(128) float wsm[];
-    float* ring = wsm + warp * NS * SLOT;
-    __shared__ float sdt[4];
-    __shared__ double red[kWalkWarps];
-    if (tid == 0) {
-        // dt from the max wave-speed sum of the step's input state (FP64, as the
-        // tiled sweep); its FP32 forms rounded here once
-        const double dt = prm.cfl / __longlong_as_double((long long)ctl->smax[prm.slot_in]);
-        sdt[0] = (float)dt;
-        sdt[1] = (float)(0.5 * dt * prm.inv_dx[AXIS]);
-        sdt[2] = (float)(0.5 / (dt * prm.inv_dx[AXIS]));  // (dx/dt)/2
-        if (blockIdx.x == 0 && prm.last) {
-            ctl->t = prm.first ? dt : ctl->t + dt;
-            ctl->dt_last = dt;
-            ctl->smax[(prm.slot_in + 2) % 3] = 0ull;
-        }
-    }
-    __syncthreads();
-    const f2 gamma = splat<f2>(prm.gamma_f), gm1 = splat<f2>(prm.gm1_f);
-    const f2 hdt = splat<f2>(sdt[1]), hidt = splat<f2>(sdt[2]);
-    const float dtf = sdt[0];
-    const f2 ndt = f2{-dtf, -dtf};
-    f2 ivx[3];
+    f2 q[DIM + 2], Fq[DIM + 2], iq, uq, pq;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) ivx[d] = splat<f2>(prm.inv_dx_f[d]);
-    const f2 iv = ivx[AXIS];
-    const int nx = g.n[0];
-    const long long cs = g.comp_stride;
-    float smax_local = 0.f;
-    bool bad = false;
+    for (int m = 0; m < DIM + 2; ++m) q[m] = fma_v(ndtdx, Fb[m] - Fa[m], a[m] + b[m]);
+    pflux<f2, DIM, D>(q, gm1, Fq, iq, uq, pq);
+#pragma unroll
+    for (int m = 0; m < DIM + 2; ++m) V[m] = fma_v(ndxdt, b[m] - a[m], (Fa[m] + Fb[m]) + Fq[m]);
+}
 
-    // Stage the chunk of 64 cells from x0 of the row whose x = 0 cell is the
-    // padded cell rb into slot s.  Slot layout: SoA component m at [64 m, 64 m
-    // + 64); AoS cell i at [NC i, NC i + NC).  A whole chunk moves as 16-byte
-    // copies coalesced across the warp (SoA: 16 per component row; AoS: the
-    // chunk's contiguous bytes, or in 2D the lane's own two cells); the lane's
-    // pieces (slot offset, source offset from the chunk's first cell) are
-    // formed once here.  A chunk past the last cell copies each lane's two
-    // cells with the index clamped to the ghost cell x = nx (never stored).
-    constexpr int NPIECE = kOwnCells ? 64 : 16 * NC;  // 16-byte pieces of a full chunk
-    constexpr int PPL = (NPIECE + 31) / 32;           // per lane
-    int pdst[PPL];
-    long long psrc[PPL];
+struct ForceConsts {
+    f2 gamma, gm1, ivx[3];
+    f2 ndtdx[3], ndxdt[3], nc[3];  // -dt/dx, -dx/dt, -(dt/dx)/4
+};
+
+// One walk: rows r0 .. r1 - 1 along axis D (1: y, 2: z) of the pair columns
+// starting at x0; XS: sweep every row along x first; LAST: the step's last
+// sweep (wave speeds, admissibility and ghost images of the new state).
+// `line` is the z plane of a y walk, the y row of a z walk.  begin() stages
+// the walk's first rows, which needs no dt; run() walks.
+template <int DIM, int LAYOUT, int D, bool XS, bool LAST>
+struct ForceWalk {
+    static constexpr int NC = DIM + 2, NS = kForceSlots, SLOT = 64 * NC;
+    static constexpr long long CST = LAYOUT == LAYOUT_SOA ? 1 : NC;
+    WalkRows rows;
+    int x0, r0, r1, line;
+    long long org, stride;
+
+    __device__ __forceinline__ void begin(const float* __restrict__ in, const WalkStep& a, int x0_, int r0_, int r1_,
+                                          int line_, float* ring, int lane)
+    {
+        const FieldGeom& g = a.g;
+        x0 = x0_; r0 = r0_; r1 = r1_; line = line_;
+        stride = (D == 1 ? g.px : g.px * g.py) * CST;
+        // element offset of x = 0 in row 0 (pairs past the field read the last pair that holds a ghost cell)
+        const long long zoff = DIM == 3 ? (long long)(g.h + (D == 1 ? line : 0)) * g.py : 0;
+        org = ((zoff + g.h + (D == 1 ? 0 : line)) * g.px + g.lead + g.h) * CST;
+        rows.init(in + org + min(x0 + 2 * lane, g.n[0] & ~1) * CST, stride, r0 - 1, g.n[D], a.bc);
+        const int n = r1 - r0 + 2;
 #pragma unroll
-    for (int t = 0; t < PPL; ++t) {
-        const int i = kOwnCells ? 2 * lane + t : lane + 32 * t;
-        if constexpr (kOwnCells) {
-            pdst[t] = 4 * i;
-            psrc[t] = (long long)i * NC;
-        } else if constexpr (LAYOUT == LAYOUT_SOA) {
-            const int m = i >> 4, part = i & 15;
-            pdst[t] = 64 * m + 4 * part;
-            psrc[t] = (long long)m * cs + 4 * part;
-        } else {
-            pdst[t] = 4 * i;
-            psrc[t] = 4LL * i;
-        }
-        if (i >= NPIECE) pdst[t] = -1;
-    }
-    auto stage = [&](float* s, long long rb, int x0) {
-        if (x0 + 64 <= nx) {
-            const float* src = LAYOUT == LAYOUT_SOA ? in + rb + x0 : in + (rb + x0) * NC;
-#pragma unroll
-            for (int t = 0; t < PPL; ++t)
-                if (t * 32 + 31 < NPIECE || pdst[t] >= 0) cp_async16(s + pdst[t], src + psrc[t]);
-        } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int c = 2 * lane + h;
-                const long long src = rb + min(x0 + c, nx);
-                if constexpr (LAYOUT == LAYOUT_SOA) {
-#pragma unroll
-                    for (int m = 0; m < NC; ++m) cp_async4(s + 64 * m + c, in + src + m * cs);
-                } else if constexpr (kOwnCells) {
-                    cp_async16(s + 4 * c, in + src * NC);
-                } else {
-#pragma unroll
-                    for (int m = 0; m < NC; ++m) cp_async4(s + NC * c + m, in + src * NC + m);
-                }
+        for (int i = 0; i < NS - 1; ++i) {
+            if (i < n) {
+                walk_stage<DIM, LAYOUT>(ring + i * SLOT, lane, rows.p, g.comp_stride);
+                rows.next();
             }
+            cp_async_commit();
         }
-    };
-    // lane 31: the cell after the chunk (the next chunk's first, or the ghost
-    // x = nx), components at [256, 260) of the slot
-    constexpr int NEXT = 64 * NC;  // offset of the cell after the chunk in a slot
-    auto stage_next = [&](float* s, long long rb, int x0) {
-        if (lane != 31) return;
-        const long long src = rb + min(x0 + 64, nx);
-        if constexpr (LAYOUT == LAYOUT_SOA) {
-#pragma unroll
-            for (int m = 0; m < NC; ++m) cp_async4(s + NEXT + m, in + src + m * cs);
-        } else if constexpr (kOwnCells) {
-            cp_async16(s + NEXT, in + src * NC);
-        } else {
-#pragma unroll
-            for (int m = 0; m < NC; ++m) cp_async4(s + NEXT + m, in + src * NC + m);
+    }
+
+    __device__ __forceinline__ void run(float* __restrict__ out, const WalkStep& a, float* ring, int lane,
+                                        const ForceConsts& k, float& smax);
+};
+
+template <int DIM, int LAYOUT, int D, bool XS, bool LAST>
+__device__ __forceinline__ void ForceWalk<DIM, LAYOUT, D, XS, LAST>::run(float* __restrict__ out, const WalkStep& a,
+                                                                        float* ring, int lane, const ForceConsts& k,
+                                                                        float& smax)
+{
+    const FieldGeom& g = a.g;
+    const int nx = g.n[0], na = g.n[D];
+    const int x = x0 + 2 * lane;
+    const bool v0 = (!XS || (lane >= 1 && lane <= 30)) && x < nx, v1 = v0 && x + 1 < nx;
+    const long long cs = g.comp_stride;
+    float* const po0 = out + org + x * CST + r0 * stride;
+    float* po = po0;
+    const int n = r1 - r0 + 2;
+    float cx = 1.f, c0 = 1.f, c1 = 1.f;  // smallest density/pressure: before the x sweep, after it (per cell)
+    WalkNew nw;
+    const bool full = x0 + 64 <= nx;  // every pair that is updated lies in the field
+    const bool edge_x = LAST && (x0 < g.h || x0 + 64 > nx - g.h);
+    const int nl = DIM == 3 ? g.n[D == 1 ? 2 : 1] : 1;  // lines across the walk's plane
+    const bool edge_l = LAST && DIM == 3 && (line < g.h || line >= nl - g.h);
+    float* rd = ring;                      // slot of row i
+    float* wr = ring + (NS - 1) * SLOT;    // slot of row i + NS - 1
+    // row i = 0 .. n - 1 of the walk (r0 - 1 + i) from the row before it: `a` holds
+    // the swept row, its flux along D and the face below it, `b` receives this row's
+    auto row = [&](int i, const f2 (&qa)[NC], const f2 (&Fa)[NC], const f2 (&Va)[NC], f2 (&qb)[NC], f2 (&Fb)[NC],
+                   f2 (&Vb)[NC]) {
+        if (i + NS - 1 < n) {
+            walk_stage<DIM, LAYOUT>(wr, lane, rows.p, cs);
+            rows.next();
         }
-    };
-    // lanes read cells that other lanes copied (see above)
-    auto ring_sync = [&]() {
-        if constexpr (!kOwnCells) __syncwarp();
-    };
-    // the lane's pair of cells (2 lane, 2 lane + 1) of a staged chunk
-    auto read_pair = [&](const float* s, f2 (&q)[NC]) {
-        if constexpr (LAYOUT == LAYOUT_SOA) {
+        cp_async_commit();
+        cp_async_wait<NS - 1>();
+        f2 ir, un, p;
+        if constexpr (XS) {
+            f2 q[NC], F[NC], b[NC], G[NC], V[NC];
+            walk_read<DIM, LAYOUT>(rd, lane, q);
+            pflux<f2, DIM, 0>(q, k.gm1, F, ir, un, p);
+            cx = min3f(cx, q[0].x, p.x);
+            cx = min3f(cx, q[0].y, p.y);
+#pragma unroll
+            for (int m = 0; m < NC; ++m) b[m] = f2{q[m].y, __shfl_down_sync(0xffffffffu, q[m].x, 1)};
+            G[0] = b[1];
+#pragma unroll
+            for (int m = 1; m < NC; ++m) G[m] = f2{F[m].y, __shfl_down_sync(0xffffffffu, F[m].x, 1)};
+            force4<DIM, 0>(q, b, F, G, k.gm1, k.ndtdx[0], k.ndxdt[0], V);
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
-                const float2 v = *reinterpret_cast<const float2*>(s + 64 * m + 2 * lane);
-                q[m] = f2{v.x, v.y};
+                const f2 Vl = f2{__shfl_up_sync(0xffffffffu, V[m].y, 1), V[m].x};
+                qb[m] = fma_v(k.nc[0], V[m] - Vl, q[m]);
             }
-        } else if constexpr (kOwnCells) {
-            const float4 A = *reinterpret_cast<const float4*>(s + 8 * lane);
-            const float4 B = *reinterpret_cast<const float4*>(s + 8 * lane + 4);
-            q[0] = f2{A.x, B.x}; q[1] = f2{A.y, B.y}; q[2] = f2{A.z, B.z}; q[3] = f2{A.w, B.w};
         } else {
-#pragma unroll
-            for (int m = 0; m < NC; ++m) q[m] = f2{s[NC * 2 * lane + m], s[NC * (2 * lane + 1) + m]};
+            walk_read<DIM, LAYOUT>(rd, lane, qb);
         }
+        pflux<f2, DIM, D>(qb, k.gm1, Fb, ir, un, p);
+        c0 = min3f(c0, qb[0].x, p.x);
+        c1 = min3f(c1, qb[0].y, p.y);
+        force4<DIM, D>(qa, qb, Fa, Fb, k.gm1, k.ndtdx[D], k.ndxdt[D], Vb);
+        if (i >= 2) {
+            f2 qn[NC];
+#pragma unroll
+            for (int m = 0; m < NC; ++m) qn[m] = fma_v(k.nc[D], Vb[m] - Va[m], qa[m]);
+            walk_store<DIM, LAYOUT>(po, cs, qn, v0, v1, full);
+            if constexpr (LAST) {
+                const int r = r0 + i - 2;
+                if (edge_x) walk_ghost_x<DIM, LAYOUT>(po, cs, qn, x, nx, g.h, a.bc, v0, v1);
+                if (r < g.h || r >= na - g.h)
+                    walk_ghost_rows<DIM, LAYOUT>(po, cs, qn, r, na, g.h, a.bc, stride, v0, v1, full);
+                if (edge_l)
+                    walk_ghost_rows<DIM, LAYOUT>(po, cs, qn, line, nl, g.h, a.bc, (D == 1 ? g.px * g.py : g.px) * CST,
+                                                 v0, v1, full);
+                nw.add<DIM>(qn, k.gamma, k.gm1, k.ivx);
+            }
+            po += stride;
+        }
+        __syncwarp();  // the lanes part at the field's edges: bring them together once a row
+        wr = rd;
+        rd = rd == ring + (NS - 1) * SLOT ? ring : rd + SLOT;
     };
-    auto load_cell = [&](long long c, float (&v)[NC]) {
-        if constexpr (LAYOUT == LAYOUT_SOA) {
+    f2 q0[NC], F0[NC], V0[NC], q1[NC], F1[NC], V1[NC];
 #pragma unroll
-            for (int m = 0; m < NC; ++m) v[m] = in[c + m * cs];
-        } else if constexpr (kOwnCells) {
-            const float4 A = *reinterpret_cast<const float4*>(in + c * NC);
-            v[0] = A.x; v[1] = A.y; v[2] = A.z; v[3] = A.w;
-        } else {
-#pragma unroll
-            for (int m = 0; m < NC; ++m) v[m] = in[c * NC + m];
-        }
-    };
-    // updated pair of cells (x, x + 1) of row (y, z): checks, CFL maximum, store, ghost images
-    auto finish = [&](const f2 (&qn)[NC], long long c, int x, int y, int z, bool v0, bool v1, bool near) {
-        // the wave speeds (and the admissibility of the new state) in the last
-        // sweep of a step only: the step's CFL maximum is that of its result,
-        // and an intermediate state reaches the next sweep's faces, whose
-        // states are checked there
-        bool ok0 = true, ok1 = true;
-        if (prm.last) {
-            const f2 sw = wave_sum2<DIM>(qn, gamma, gm1, ivx, ok0, ok1);
-            smax_local = fmaxf(smax_local, fmaxf(v0 ? sw.x : 0.f, v1 ? sw.y : 0.f));
-        }
-        const bool b0 = v0 && !ok0, b1 = v1 && !ok1;
-        // warp-uniform branches around the rare paths (a non-admissible cell, a
-        // ragged last chunk), so the common path has no divergent region
-        if (__any_sync(0xffffffffu, b0 || b1)) {
-            if (b0 || b1) {
-                bad = true;
-                record_bad(ctl, BAD_CELL, b0 ? x : x + 1, y, z);
-            }
-        }
-        if (__all_sync(0xffffffffu, v0 && v1) || (v0 && v1)) {
-            if constexpr (LAYOUT == LAYOUT_SOA) {
-#pragma unroll
-                for (int m = 0; m < NC; ++m)
-                    *reinterpret_cast<float2*>(out + c + m * cs) = make_float2(qn[m].x, qn[m].y);
-            } else if constexpr (kOwnCells) {
-                *reinterpret_cast<float4*>(out + c * NC) = make_float4(qn[0].x, qn[1].x, qn[2].x, qn[3].x);
-                *reinterpret_cast<float4*>(out + c * NC + NC) = make_float4(qn[0].y, qn[1].y, qn[2].y, qn[3].y);
-            } else {
-#pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    out[c * NC + m] = qn[m].x;
-                    out[(c + 1) * NC + m] = qn[m].y;
-                }
-            }
-        } else if (v0) {
-#pragma unroll
-            for (int m = 0; m < NC; ++m) out[c * g.cell_stride + m * cs] = qn[m].x;
-        }
-        if (near) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (!(h == 0 ? v0 : v1)) continue;
-                float q1[NC];
-#pragma unroll
-                for (int m = 0; m < NC; ++m) q1[m] = h == 0 ? qn[m].x : qn[m].y;
-                write_ghost_images<float, DIM>(out, g, prm.bc, x + h, y, z, q1);
-            }
-        }
-    };
-    // padded cell index of cell (0, y, z)
-    auto row_base = [&](int y, int z) -> long long {
-        return ((long long)(DIM == 3 ? g.h + z : 0) * g.py + (g.h + y)) * g.px + g.lead + g.h;
-    };
-
-    // x sweep: the face xs - 1/2 that starts each walk, for 32 of the warp's
-    // walks at a time (lane j: the warp's walk jb + j), in the packed
-    // arithmetic of the walk before, which gives the same bits: the two walks
-    // agree on their common face exactly.  One evaluation per 32 walks instead
-    // of one per walk (a 256-cell row is a walk of only four chunks).
-    const int wstride = gridDim.x * kWalkWarps;
-    float bface[NC];
-    float bchk = 1.f;
-    int jw = 0;  // walks of this warp so far
-    for (int w = blockIdx.x * kWalkWarps + warp; w < wg.walks; w += wstride, ++jw) {
-        float chk = 1.f;
-        int wx, wy, wz = 0;  // first cell of the walk (reported with a non-admissible face state)
-        ring_sync();  // the previous walk's reads of the ring come before its refill
-        if constexpr (AXIS == 0) {
-            const int r = w / wg.nseg, xs = (w % wg.nseg) * wg.seg;
-            const int y = r % g.n[1], z = r / g.n[1];
-            const int xe = min(xs + wg.seg, nx);
-            const int nch = (xe - xs + 63) >> 6;
-            const long long rb = row_base(y, z);  // padded cell of x = 0
-            const bool row_near = y < g.h || y >= g.n[1] - g.h || (DIM == 3 && (z < g.h || z >= g.n[2] - g.h));
-            wx = xs;
-            wy = y;
-            wz = z;
-            // chunk k in slot k % NS, staged NS - 1 chunks ahead (one copy group per chunk)
-#pragma unroll
-            for (int k = 0; k < NS - 1; ++k) {
-                if (k < nch) {
-                    stage(ring + k * SLOT, rb, xs + 64 * k);
-                    stage_next(ring + k * SLOT, rb, xs + 64 * k);
-                }
-                cp_async_commit();
-            }
-            // face xs - 1/2, the left face of lane 0's first chunk
-            if ((jw & 31) == 0) {
-                const int wl = w + lane * wstride;  // this lane's walk of the batch
-                const int rl = min(wl, wg.walks - 1) / wg.nseg, xl = (min(wl, wg.walks - 1) % wg.nseg) * wg.seg;
-                const long long rbl = row_base(rl % g.n[1], rl / g.n[1]);
-                float l[NC], r[NC];
-                load_cell(rbl + xl - 1, l);
-                load_cell(rbl + xl, r);
-                f2 a[NC], b[NC], F[NC];
-#pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    a[m] = splat<f2>(l[m]);
-                    b[m] = splat<f2>(r[m]);
-                }
-                bchk = 1.f;
-                force<f2, DIM, 0>(a, b, gm1, hdt, hidt, F, bchk);
-#pragma unroll
-                for (int m = 0; m < NC; ++m) bface[m] = F[m].x;
-            }
-            float carry[NC];
-#pragma unroll
-            for (int m = 0; m < NC; ++m) carry[m] = __shfl_sync(0xffffffffu, bface[m], jw & 31);
-            chk = __shfl_sync(0xffffffffu, bchk, jw & 31);
-            int slot = 0;  // slot of chunk k
+    for (int m = 0; m < NC; ++m) q0[m] = F0[m] = V0[m] = f2{1.f, 1.f};  // the first face of a walk is not used
+    // two rows per iteration, so that what passes from row to row changes hands without copies
 #pragma unroll 1
-            for (int k = 0; k < nch; ++k) {
-                const int x0 = xs + (k << 6), x = x0 + 2 * lane;
-                {
-                    // refill the slot read in the previous iteration with chunk k + NS - 1
-                    const int kn = k + NS - 1;
-                    float* s = ring + (slot == 0 ? NS - 1 : slot - 1) * SLOT;
-                    ring_sync();
-                    if (kn < nch) {
-                        stage(s, rb, xs + 64 * kn);
-                        stage_next(s, rb, xs + 64 * kn);
-                    }
-                    cp_async_commit();
-                }
-                cp_async_wait<NS - 1>();  // chunk k has landed
-                ring_sync();
-                const float* s = ring + slot * SLOT;
-                f2 q[NC], b[NC], Fr[NC], qn[NC];
-                read_pair(s, q);
-                // right faces of the lane's cells: (x | x + 1) and (x + 1 | x + 2)
-#pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    float rn = __shfl_down_sync(0xffffffffu, q[m].x, 1);
-                    if (lane == 31) rn = s[NEXT + m];
-                    b[m] = f2{q[m].y, rn};
-                }
-                force<f2, DIM, 0>(q, b, gm1, hdt, hidt, Fr, chk);
-#pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    float fl = __shfl_up_sync(0xffffffffu, Fr[m].y, 1);
-                    if (lane == 0) fl = carry[m];
-                    carry[m] = __shfl_sync(0xffffffffu, Fr[m].y, 31);
-                    qn[m] = fma_v(ndt, (Fr[m] - f2{fl, Fr[m].x}) * iv, q[m]);
-                }
-                finish(qn, rb + x, x, y, z, x < xe, x + 1 < xe, row_near || x0 < g.h || x0 + 64 > nx - g.h);
-                slot = slot == NS - 1 ? 0 : slot + 1;
-            }
-        } else {
-            // walk: strip of columns x0 .. x0 + 63, line (z for a y sweep, y for a z
-            // sweep), rows ys .. ye - 1 along the swept axis
-            const int na = g.n[AXIS];
-            const int strip = w % wg.nstrips, rest = w / wg.nstrips;
-            const int line = rest % wg.nlines, ys = (rest / wg.nlines) * wg.seg;
-            const int ye = min(ys + wg.seg, na);
-            const int x0 = strip << 6, x = x0 + 2 * lane;
-            const bool v0 = x < nx, v1 = x + 1 < nx;
-            const int nl = DIM == 3 ? g.n[AXIS == 1 ? 2 : 1] : 1;
-            const bool col_near = x0 < g.h || x0 + 64 > nx - g.h || (DIM == 3 && (line < g.h || line >= nl - g.h));
-            const long long stride = AXIS == 1 ? g.px : g.px * g.py;
-            const long long base = AXIS == 1 ? row_base(0, line) : row_base(line, 0);  // padded cell of (0, row 0)
-            auto coords = [&](int row, int& y, int& z) {
-                y = AXIS == 1 ? row : line;
-                z = AXIS == 1 ? line : row;
-            };
-            wx = x0;
-            coords(ys, wy, wz);
-            // row ys - 1 + i in slot i % NS, i = 0 .. ye - ys + 1 (rows ys - 1 and ye
-            // are ghost rows at the field's edges), staged NS - 2 rows ahead
-            const int nrows = ye - ys + 2;
-#pragma unroll
-            for (int i = 0; i < NS - 1; ++i) {
-                if (i < nrows) stage(ring + i * SLOT, base + (long long)(ys - 1 + i) * stride, x0);
-                cp_async_commit();
-            }
-            cp_async_wait<NS - 3>();  // rows ys - 1 and ys
-            ring_sync();
-            f2 Fl[NC];  // face below row r (between rows r - 1 and r)
-            {
-                f2 up[NC], q0[NC];
-                read_pair(ring, up);
-                read_pair(ring + SLOT, q0);
-                force<f2, DIM, AXIS>(up, q0, gm1, hdt, hidt, Fl, chk);
-            }
-            int slot = 1;  // slot of row r
-            long long rb_next = base + (long long)(ys + NS - 2) * stride;  // row ys - 1 + (i + NS - 2)
-            long long c_row = base + (long long)ys * stride + x;            // the lane's first cell of row r
-#pragma unroll 1
-            for (int r = ys; r < ye; ++r, rb_next += stride, c_row += stride) {
-                const int i = r - ys + 1;
-                {
-                    // refill the slot of row i - 2 (read in the previous iteration) with row i + NS - 2
-                    const int ir = i + NS - 2;
-                    const int sr = slot >= 2 ? slot - 2 : slot + NS - 2;
-                    ring_sync();
-                    if (ir < nrows) stage(ring + sr * SLOT, rb_next, x0);
-                    cp_async_commit();
-                }
-                cp_async_wait<NS - 3>();  // rows r and r + 1
-                ring_sync();
-                const int sn = slot == NS - 1 ? 0 : slot + 1;
-                f2 q[NC], qd[NC], Fr[NC], qn[NC];
-                read_pair(ring + slot * SLOT, q);
-                read_pair(ring + sn * SLOT, qd);
-                force<f2, DIM, AXIS>(q, qd, gm1, hdt, hidt, Fr, chk);
-#pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    qn[m] = fma_v(ndt, (Fr[m] - Fl[m]) * iv, q[m]);
-                    Fl[m] = Fr[m];
-                }
-                int y, z;
-                coords(r, y, z);
-                finish(qn, c_row, x, y, z, v0, v1, col_near || r < g.h || r >= na - g.h);
-                slot = sn;
-            }
-        }
-        if (!(chk > 0.f)) {
-            bad = true;
-            record_bad(ctl, BAD_STATE, wx, wy, wz);
-        }
+    for (int i = 0; i < n; i += 2) {
+        row(i, q0, F0, V0, q1, F1, V1);
+        if (i + 1 >= n) break;
+        row(i + 1, q1, F1, V1, q0, F0, V0);
     }
-    cp_async_wait<0>();
+    if constexpr (LAST) smax = fmaxf(smax, fmaxf(v0 ? nw.s0 : 0.f, v1 ? nw.s1 : 0.f));
+    // a non-admissible state on some face of the walk (columns outside the
+    // walk or the field are copies, padding (NaN) or undefined after the sweep)
+    if ((XS && !(cx > 0.f)) || (v0 && !(c0 > 0.f)) || (v1 && !(c1 > 0.f))) {
+        record_bad(a.ctl, BAD_STATE, max(x, 0), D == 1 ? r0 : line, D == 1 ? line : r0);
+        atomicOr(&a.ctl->err, DEV_ERR_NUMERIC);
+    }
+    if constexpr (LAST) {
+        const long long cstr = LAYOUT == LAYOUT_SOA ? cs : 1;
+        if (v0 && !nw.ok0) walk_bad_cell<DIM>(&a, po0, stride, cstr, D, x, line, r0, r1);
+        if (v1 && !nw.ok1) walk_bad_cell<DIM>(&a, po0 + CST, stride, cstr, D, x + 1, line, r0, r1);
+    }
+}
 
-    double v = (double)smax_local;
+template <int DIM, int LAYOUT>
+__global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_force_walk_kernel(const __grid_constant__ WalkStep a)
+{
+    constexpr int NC = DIM + 2;
+    extern __shared__ __align__(128) float wsm[];
+    __shared__ float sdt[9];
+    __shared__ float red[kWalkWarps];
+    __shared__ int sflag[1];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    float* ring = wsm + warp * kForceSlots * 64 * NC;
+    FieldCtl* ctl = a.ctl;
+    ForceConsts k;
+    k.gamma = splat<f2>(a.gamma_f);
+    k.gm1 = splat<f2>(a.gm1_f);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int any_bad = __syncthreads_or(bad ? 1 : 0);
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    if (tid == 0) {
-        double m = 0.0;
-        for (int k = 0; k < kWalkWarps; ++k) m = fmax(m, red[k]);
-        if (prm.last) atomic_max_pos_double(&ctl->smax[(prm.slot_in + 1) % 3], m);
-        if (any_bad) atomicOr(&ctl->err, DEV_ERR_NUMERIC);
+    for (int d = 0; d < 3; ++d) k.ivx[d] = splat<f2>(a.inv_dx_f[d]);
+    if (tid == 0) sflag[0] = 0;
+    unsigned phase = 0;  // a barrier ends every phase but the last
+    for (int s = 0; s < a.K; ++s) {
+        const int rs = (a.slot + s) % 3;
+        const int cur = DIM == 3 ? a.cur : (a.cur + s) & 1;
+        float* A = a.buf[cur];
+        float* B = a.buf[cur ^ 1];
+        ForceWalk<DIM, LAYOUT, 1, true, DIM == 2> w;
+        const int per = a.strips * a.segs;
+        WalkUnits todo(ctl, phase, DIM == 3 ? per * a.g.n[2] : per, lane, warp);
+        auto begin = [&]() {
+            if (!todo.any()) return;
+            const int pl = DIM == 3 ? todo.u / per : 0, v = DIM == 3 ? todo.u % per : todo.u;
+            const int strip = v % a.strips, r0 = (v / a.strips) * a.rows;
+            w.begin(A, a, strip * kWalkUse - 2, r0, min(a.g.n[1], r0 + a.rows), pl, ring, lane);
+        };
+        begin();
+        if (tid == 0) {
+            // dt from the largest wave-speed sum of the step's input state, in FP64 once per CTA
+            const double sm = __longlong_as_double((long long)__ldcg(&ctl->smax[rs]));
+            const double dt = a.cfl / sm;
+            for (int d = 0; d < DIM; ++d) {
+                sdt[d] = (float)(-dt * a.inv_dx[d]);
+                sdt[3 + d] = (float)(-sm * a.dx_cfl[d]);
+                sdt[6 + d] = (float)(-0.25 * dt * a.inv_dx[d]);
+            }
+            if (blockIdx.x == 0) {
+                ctl->t = s == 0 && a.first ? dt : ctl->t + dt;
+                ctl->dt_last = dt;
+                ctl->smax[(rs + 2) % 3] = 0ull;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+            k.ndtdx[d] = splat<f2>(sdt[d]);
+            k.ndxdt[d] = splat<f2>(sdt[3 + d]);
+            k.nc[d] = splat<f2>(sdt[6 + d]);
+        }
+        float smax = 0.f;
+        while (todo.any()) {
+            todo.ask();
+            w.run(B, a, ring, lane, k, smax);
+            todo.advance();
+            begin();
+        }
+        if constexpr (DIM == 3) {
+            if (!walk_barrier(ctl, ++phase, a.spin_limit, sflag)) break;
+            const int zper = a.zstrips * a.g.n[1];
+            ForceWalk<DIM, LAYOUT, DIM - 1, false, true> wz;
+            for (WalkUnits zt(ctl, phase, zper * a.zsegs, lane, warp); zt.any(); zt.advance()) {
+                zt.ask();
+                const int v = zt.u % zper, r0 = (zt.u / zper) * a.zrows;
+                wz.begin(B, a, (v % a.zstrips) * 64, r0, min(a.g.n[2], r0 + a.zrows), v / a.zstrips, ring, lane);
+                wz.run(A, a, ring, lane, k, smax);
+            }
+        }
+        walk_reduce(ctl, (rs + 1) % 3, smax, red);
+        if (s + 1 < a.K && !walk_barrier(ctl, ++phase, a.spin_limit, sflag)) break;
     }
+    if (sflag[0]) {
+        if (tid == 0) atomicOr(&ctl->err, DEV_ERR_TIMEOUT);
+        return;
+    }
+    walk_leave(ctl);
 }
 
 }  // namespace ripple
@@ -439,34 +294,25 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2)
 
 namespace ripple {
 
-// Host launch helpers of the walk sweeps (one instantiation per dim, layout, axis).
-template <int DIM, int LAYOUT, int AXIS>
-static cudaError_t walk_configure()
+template <int DIM, int LAYOUT>
+static int force_walk_occupancy()  // resident CTAs per SM, 0 if the kernel cannot run
 {
-    static cudaError_t e = cudaFuncSetAttribute(euler_force_walk_kernel<DIM, LAYOUT, AXIS, kWalkSlots>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                WalkCfg<DIM, kWalkSlots>::SMEM);
-    return e;
-}
-template <int DIM, int LAYOUT, int AXIS>
-static cudaError_t walk_launch(const WalkLaunch& L)
-{
-    const cudaError_t e = walk_configure<DIM, LAYOUT, AXIS>();
-    if (e != cudaSuccess) return e;
-    euler_force_walk_kernel<DIM, LAYOUT, AXIS, kWalkSlots>
-        <<<L.grid, kWalkWarps * 32, WalkCfg<DIM, kWalkSlots>::SMEM, L.stream>>>(
-            static_cast<const float*>(L.in), static_cast<float*>(L.out), L.ctl, L.wg, L.prm);
-    return cudaGetLastError();
-}
-template <int DIM, int LAYOUT, int AXIS>
-static int walk_occ()
-{
-    if (walk_configure<DIM, LAYOUT, AXIS>() != cudaSuccess) return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, euler_force_walk_kernel<DIM, LAYOUT, AXIS, kWalkSlots>,
-                                                      kWalkWarps * 32, WalkCfg<DIM, kWalkSlots>::SMEM) != cudaSuccess)
-        return 0;
+    static const int n = [] {
+        auto kern = euler_force_walk_kernel<DIM, LAYOUT>;
+        int c = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, force_smem<DIM>()) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, kWalkWarps * 32, force_smem<DIM>()) != cudaSuccess)
+            return 0;
+        return c;
+    }();
     return n;
+}
+template <int DIM, int LAYOUT>
+static cudaError_t force_walk_run(const WalkStep& a, int grid, cudaStream_t s)
+{
+    void* args[] = {const_cast<WalkStep*>(&a)};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(euler_force_walk_kernel<DIM, LAYOUT>), dim3(grid),
+                                       dim3(kWalkWarps * 32), args, force_smem<DIM>(), s);
 }
 
 }  // namespace ripple

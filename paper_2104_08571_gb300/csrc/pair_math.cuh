@@ -115,6 +115,13 @@ __device__ __forceinline__ void track4(float& chk, f2 a, f2 b, f2 c, f2 d)
     chk = min3f(chk, min3f(m0, m1, d.x), d.y);
 }
 
+// The same with a minimum per lane, where the two cells count separately.
+__device__ __forceinline__ void track4(f2& chk, f2 a, f2 b, f2 c, f2 d)
+{
+    chk.x = min3f(chk.x, min3f(a.x, b.x, c.x), d.x);
+    chk.y = min3f(chk.y, min3f(a.y, b.y, c.y), d.y);
+}
+
 // Physical flux along axis D; also returns 1/rho, the normal velocity, the pressure.
 template <typename V, int DIM, int D>
 __device__ __forceinline__ void pflux(const V (&q)[DIM + 2], V gm1, V (&F)[DIM + 2], V& inv_rho, V& un, V& p)
@@ -129,6 +136,16 @@ __device__ __forceinline__ void pflux(const V (&q)[DIM + 2], V gm1, V (&F)[DIM +
 #pragma unroll
     for (int e = 0; e < DIM; ++e) F[1 + e] = e == D ? fma_v(q[1 + e], un, p) : q[1 + e] * un;
     F[DIM + 1] = (q[DIM + 1] + p) * un;
+}
+
+// The y flux of a 2D state whose 1/rho and pressure are known.
+__device__ __forceinline__ void pflux_y(const f2 (&q)[4], f2 inv_rho, f2 p, f2 (&F)[4], f2& v)
+{
+    v = q[2] * inv_rho;
+    F[0] = q[2];
+    F[1] = q[1] * v;
+    F[2] = fma_v(q[2], v, p);
+    F[3] = (q[3] + p) * v;
 }
 
 // Wave-speed sums sum_d (|u_d| + c)/dx_d of a pair of conserved states and
@@ -171,6 +188,20 @@ __device__ __forceinline__ void rus(const V (&a)[DIM + 2], const V (&b)[DIM + 2]
     for (int m = 0; m < DIM + 2; ++m) F[m] = half * fma_v(s, a[m] - b[m], Fa[m] + Fb[m]);
 }
 
+// Twice the Rusanov flux, the admissibility of its states per lane.
+template <int DIM, int D>
+__device__ __forceinline__ void rus2(const f2 (&a)[DIM + 2], const f2 (&b)[DIM + 2], f2 gamma, f2 gm1,
+                                     f2 (&V)[DIM + 2], f2& chk)
+{
+    f2 Fa[DIM + 2], Fb[DIM + 2], ia, ua, pa, ib, ub, pb;
+    pflux<f2, DIM, D>(a, gm1, Fa, ia, ua, pa);
+    pflux<f2, DIM, D>(b, gm1, Fb, ib, ub, pb);
+    track4(chk, a[0], pa, b[0], pb);
+    const f2 s = max_v(abs_v(ua) + sqrt_v(gamma * pa * ia), abs_v(ub) + sqrt_v(gamma * pb * ib));
+#pragma unroll
+    for (int m = 0; m < DIM + 2; ++m) V[m] = fma_v(s, a[m] - b[m], Fa[m] + Fb[m]);
+}
+
 // FORCE face flux along D (Toro): the mean of the Lax-Friedrichs flux and
 // the flux of the Richtmyer state q = (a + b)/2 - (dt/dx)/2 (F(b) - F(a));
 // dtdx = dt/dx, inv_dtdx = dx/dt.  Admissibility of a and b goes to chk (q is
@@ -193,9 +224,9 @@ __device__ __forceinline__ void force(const V (&a)[DIM + 2], const V (&b)[DIM + 
 }
 
 // MUSCL-Hancock face states of cells along D from (left, centre, right).
-template <typename V, int DIM, int D>
+template <typename V, int DIM, int D, typename C>
 __device__ __forceinline__ void muscl(const V (&qm)[DIM + 2], const V (&q)[DIM + 2], const V (&qp)[DIM + 2], V gm1,
-                                      V half_dtdx, V (&L)[DIM + 2], V (&R)[DIM + 2], float& chk)
+                                      V half_dtdx, V (&L)[DIM + 2], V (&R)[DIM + 2], C& chk)
 {
     const V half = splat<V>(0.5f), mhalf = splat<V>(-0.5f);
 #pragma unroll

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <string>
 
+#include "grid_sync.cuh"
 #include "runtime.h"
 
 namespace ripple {
@@ -278,7 +279,10 @@ ripple_status take_device_error(ripple_field f)
     unsigned err = 0;
     RIPPLE_CUDA(cudaMemcpyAsync(&err, &f->ctl->err, sizeof(unsigned), cudaMemcpyDeviceToHost, f->ctx->stream));
     RIPPLE_CUDA(cudaStreamSynchronize(f->ctx->stream));
-    if (err) RIPPLE_CUDA(cudaMemsetAsync(&f->ctl->err, 0, sizeof(unsigned), f->ctx->stream));
+    if (err) {
+        RIPPLE_CUDA(cudaMemsetAsync(&f->ctl->err, 0, sizeof(unsigned), f->ctx->stream));
+        RIPPLE_CUDA(cudaMemsetAsync(f->ctl->bar, 0, sizeof(f->ctl->bar) + sizeof(f->ctl->work), f->ctx->stream));
+    }
     return map_dev_err(err);
 }
 
@@ -566,37 +570,94 @@ ripple_status ripple_field_set_sweep(ripple_field f, int variant, int zchunk)
     return RIPPLE_OK;
 }
 
-// Walks of a one-axis sweep (euler_force_walk.cuh): about 16 per resident
-// warp, so that the grid-stride walks spread evenly over the SMs, and at least
-// 4 chunks (x) or 16 rows (y, z) long, so that the face a walk shares with the
-// walk before it (evaluated by both) stays a small part of the arithmetic.
-static WalkGeom walk_geom(const FieldGeom& g, int axis, long long resident_warps)
+// Rows per walk for `lines` independent lines of n rows on `sms` SMs of 16
+// resident warps, a walk of R rows costing R + extra.  In units of the time a
+// warp alone takes for a row, a scheduler with enough warps finishes a row
+// every 0.28 (a warp issues about every fourth cycle).  Walks that all have a
+// warp of their own end together; otherwise the last one handed out ends about
+// 0.6 walks after the schedulers have run out of others.  `most` bounds R:
+// walks along z keep as many planes in flight as they are long and lose L2
+// hits (200 x 171 x 186: 8 planes 149 us a step, 31 190, 62 223), and long
+// in-plane walks of a 3D field do the same (24 rows).
+static void walk_split(long long lines, int n, int sms, double extra, int most, int* rows, int* segs)
 {
-    WalkGeom w{};
-    w.f = g;
-    const long long target = std::max(1LL, 16 * resident_warps);
-    const long long nch = (g.n[0] + 63) / 64;
-    const long long nyz = (long long)g.n[1] * (g.ndim == 3 ? g.n[2] : 1);  // rows of the x sweep
-    if (axis == 0) {
-        long long cpw = nch * nyz / target;
-        cpw = std::max(std::min(cpw, nch), std::min(4LL, nch));
-        w.seg = (int)(64 * cpw);
-        w.nseg = (int)((nch + cpw - 1) / cpw);
-        w.nstrips = 0;
-        w.nlines = 1;
-        w.walks = (int)(w.nseg * nyz);
-    } else {
-        const long long na = g.n[axis];
-        const long long lines = g.ndim == 3 ? g.n[axis == 1 ? 2 : 1] : 1;
-        long long rows = nch * lines * na / target;
-        rows = std::max(std::min(rows, na), std::min(16LL, na));
-        w.seg = (int)rows;
-        w.nseg = (int)((na + rows - 1) / rows);
-        w.nstrips = (int)nch;
-        w.nlines = (int)lines;
-        w.walks = (int)(w.nseg * nch * lines);
+    double best = 1e300;
+    *rows = n;
+    *segs = 1;
+    for (int r = 1; r <= std::min(n, most); ++r) {
+        const int sg = (n + r - 1) / r;
+        const long long units = lines * sg, per = (units + 4 * sms - 1) / (4 * sms);  // walks per scheduler
+        const double cost = units <= (long long)kWalkWarps * sms
+                                ? (r + extra) * std::max(1.0, 0.28 * (double)per)
+                                : (r + extra) * ((double)units * 0.28 / (4.0 * sms) + 0.6);
+        if (cost < best) {
+            best = cost;
+            *rows = r;
+            *segs = sg;
+        }
     }
-    return w;
+}
+
+// Steps of a walk launch: about 64 M cell updates, so that a launch stays near
+// a millisecond (a long call is then cut into several launches).
+static int walk_steps(const FieldGeom& g, int64_t left)
+{
+    const long long cells = (long long)g.n[0] * g.n[1] * g.n[2];
+    return (int)std::min<long long>(left, std::max(1LL, std::min(256LL, (64LL << 20) / cells)));
+}
+
+// Steps of an FP32 field on strip walks: every 2D scheme, and the split FORCE
+// step in 3D.
+static ripple_status walk_field_steps(ripple_field U, const SweepParams& prm, int scheme, int layout, int64_t nsteps)
+{
+    ripple_ctx ctx = U->ctx;
+    const FieldGeom& g = U->geom;
+    const bool force = scheme == SCHEME_FORCE;
+    const bool d3 = U->ndim == 3;  // FORCE only
+    const int occ = d3      ? force_walk_occ_f32_3d(layout)
+                    : force ? force_walk_occ_f32_2d(layout)
+                            : walk2d_occ_f32(scheme, layout);
+    if (occ <= 0) return fail(RIPPLE_ERR_INTERNAL, "walk kernel does not fit");
+    const int ctas = occ * ctx->sm_count;
+    WalkStep a{};
+    a.buf[0] = static_cast<float*>(U->buf[0]);
+    a.buf[1] = static_cast<float*>(U->buf[1]);
+    a.ctl = U->ctl;
+    a.g = g;
+    a.cfl = prm.cfl;
+    a.gamma_f = prm.gamma_f;
+    a.gm1_f = prm.gm1_f;
+    for (int d = 0; d < 3; ++d) {
+        a.inv_dx[d] = prm.inv_dx[d];
+        a.dx_cfl[d] = prm.inv_dx[d] > 0.0 ? 1.0 / (prm.inv_dx[d] * prm.cfl) : 0.0;
+        a.inv_dx_f[d] = prm.inv_dx_f[d];
+    }
+    a.bc = prm.bc;
+    a.spin_limit = grid_spin_limit();
+    a.strips = (g.n[0] + kWalkUse - 1) / kWalkUse;
+    walk_split((long long)a.strips * g.n[2], g.n[1], ctx->sm_count,
+               scheme == SCHEME_RUSANOV1 ? 1.5 : 2.0, d3 ? 24 : 128, &a.rows, &a.segs);
+    long long units = (long long)a.strips * a.segs * g.n[2];
+    if (d3) {
+        a.zstrips = (g.n[0] + 63) / 64;
+        walk_split((long long)a.zstrips * g.n[1], g.n[2], ctx->sm_count, 1.0, 8, &a.zrows, &a.zsegs);
+        units = std::max(units, (long long)a.zstrips * g.n[1] * a.zsegs);
+    }
+    // unit numbers are 32-bit: at most 2^32 padded cells and at least 60 cells per unit row
+    const int grid = (int)std::min<long long>(ctas, units);
+    for (int64_t done = 0; done < nsteps;) {
+        a.K = walk_steps(g, nsteps - done);
+        a.cur = U->cur;
+        a.slot = (int)(U->steps_total % 3);
+        a.first = done == 0;
+        RIPPLE_CUDA(d3      ? force_walk_launch_f32_3d(layout, a, grid, ctx->stream)
+                    : force ? force_walk_launch_f32_2d(layout, a, grid, ctx->stream)
+                            : walk2d_launch_f32(scheme, layout, a, grid, ctx->stream));
+        if (!d3) U->cur = (U->cur + a.K) & 1;  // 3D: the z walks bring the state back
+        U->steps_total += a.K;
+        done += a.K;
+    }
+    return RIPPLE_OK;
 }
 
 ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t nsteps, ripple_fv_stats* stats)
@@ -731,36 +792,17 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     // one launch per step (unsplit), or one sweep per axis (split: x, then y, then z;
     // each sweep writes the ghost images its successor reads; all read the same dt)
     const int sweeps = split ? U->ndim : 1;
-    // the split step of an FP32 field sweeps on strip walks (no tile staging)
-    const bool walk = split && U->dtype == RIPPLE_F32 && U->variant < 0;
-    WalkLaunch W[3]{};
-    if (walk) {
-        for (int a = 0; a < U->ndim; ++a) {
-            const int wocc = U->ndim == 2 ? force_walk_occ_f32_2d(layout, a) : force_walk_occ_f32_3d(layout, a);
-            if (wocc <= 0) return fail(RIPPLE_ERR_INTERNAL, "walk sweep kernel does not fit");
-            W[a].wg = walk_geom(g, a, (long long)wocc * ctx->sm_count * kWalkWarps);
-            W[a].grid = (int)std::min<long long>((W[a].wg.walks + kWalkWarps - 1) / kWalkWarps,
-                                                 (long long)wocc * ctx->sm_count);
-            W[a].ctl = U->ctl;
-            W[a].stream = s;
-            W[a].prm = L.prm;
-        }
+    int64_t nsteps_left = nsteps;
+    // FP32 fields: the 2D schemes and the split step run on strip walks (no
+    // tile staging, several steps per launch) unless a kernel was chosen
+    if (U->dtype == RIPPLE_F32 && U->variant < 0 && (U->ndim == 2 || split)) {
+        st = walk_field_steps(U, L.prm, scheme, layout, nsteps);
+        if (st != RIPPLE_OK) return st;
+        nsteps_left = 0;
     }
-    for (int64_t n = 0; n < nsteps; ++n) {
+    for (int64_t n = 0; n < nsteps_left; ++n) {
         for (int a = 0; a < sweeps; ++a) {
             const int in = U->cur, outb = 1 - U->cur;
-            if (walk) {
-                W[a].in = U->buf[in];
-                W[a].out = U->buf[outb];
-                W[a].prm.slot_in = (int)(U->steps_total % 3);
-                W[a].prm.first = n == 0;
-                W[a].prm.axis = a;
-                W[a].prm.last = a == sweeps - 1;
-                RIPPLE_CUDA(U->ndim == 2 ? force_walk_launch_f32_2d(layout, a, W[a])
-                                         : force_walk_launch_f32_3d(layout, a, W[a]));
-                U->cur = outb;
-                continue;
-            }
             // the row kernel stages AoS planes through the grouped view and
             // stores its results directly (no output map)
             const bool rowk = v == kRowVariant;
@@ -803,6 +845,7 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     if (host.err) {
         RIPPLE_CUDA(cudaMemsetAsync(&U->ctl->err, 0, sizeof(unsigned), s));
         RIPPLE_CUDA(cudaMemsetAsync(&U->ctl->counters[4], 0, 4 * sizeof(long long), s));
+        RIPPLE_CUDA(cudaMemsetAsync(U->ctl->bar, 0, sizeof(U->ctl->bar) + sizeof(U->ctl->work), s));  // after a wait that ran out
         return map_dev_err(host.err, &host);
     }
     return RIPPLE_OK;

@@ -15,6 +15,7 @@
 #include "../../include/ripple.h"
 #include "euler_sweep.cuh"
 #include "field.cuh"
+#include "walk_common.cuh"
 
 namespace ripple {
 
@@ -86,23 +87,16 @@ int sweep_occ_f32_3d(int layout, int scheme, int v);
 int sweep_occ_f64_2d(int layout, int scheme, int v);
 int sweep_occ_f64_3d(int layout, int scheme, int v);
 
-// One sweep of the split FORCE step of an FP32 field on strip walks
-// (euler_force_walk.cuh), along axis 0, 1 (or 2 in 3D); defined with the FP32
-// sweeps of the same dimension.
-struct WalkLaunch {
-    const void* in;
-    void* out;
-    FieldCtl* ctl;
-    WalkGeom wg;
-    SweepParams prm;
-    int grid;
-    cudaStream_t stream;
-};
-cudaError_t force_walk_launch_f32_2d(int layout, int axis, const WalkLaunch& L);
-cudaError_t force_walk_launch_f32_3d(int layout, int axis, const WalkLaunch& L);
-// Resident CTAs per SM of the walk kernel (0 on error).
-int force_walk_occ_f32_2d(int layout, int axis);
-int force_walk_occ_f32_3d(int layout, int axis);
+// Steps of the split FORCE solver of an FP32 field on strip walks
+// (euler_force_walk.cuh): one cooperative launch of `grid` CTAs, at most the
+// resident CTAs per SM (force_walk_occ_*, 0 on error) times the SMs.
+cudaError_t force_walk_launch_f32_2d(int layout, const WalkStep& a, int grid, cudaStream_t s);
+cudaError_t force_walk_launch_f32_3d(int layout, const WalkStep& a, int grid, cudaStream_t s);
+int force_walk_occ_f32_2d(int layout);
+int force_walk_occ_f32_3d(int layout);
+// The same for the FP32 2D unsplit schemes (euler_walk2d.cuh), one launch for several steps.
+cudaError_t walk2d_launch_f32(int scheme, int layout, const WalkStep& a, int grid, cudaStream_t s);
+int walk2d_occ_f32(int scheme, int layout);
 
 // Aux kernels (f32/f64 x 2D/3D), defined in aux.cu.
 cudaError_t launch_prep(int dtype, int dim, void* buf, FieldCtl* ctl, const FieldGeom& g, int bc, double gamma,

@@ -1,6 +1,7 @@
 // Euler sweep kernels, element type float, 2D (all layouts, schemes, tiles),
-// and the strip-walk sweeps of the split FORCE step.
+// and the strip walks of the split FORCE step.
 #include "euler_force_walk.cuh"
+#include "euler_walk2d.cuh"
 #include "sweep_table.cuh"
 
 namespace ripple {
@@ -11,15 +12,29 @@ cudaError_t sweep_launch_f32_2d(int layout, int scheme, int v, const SweepLaunch
 int sweep_smem_f32_2d(int layout, int scheme, int v) { return SweepDim<float, 2>::smem(layout, scheme, v); }
 int sweep_occ_f32_2d(int layout, int scheme, int v) { return SweepDim<float, 2>::occ(layout, scheme, v); }
 
-cudaError_t force_walk_launch_f32_2d(int layout, int axis, const WalkLaunch& L)
+cudaError_t force_walk_launch_f32_2d(int layout, const WalkStep& a, int grid, cudaStream_t s)
 {
-    if (axis != 0 && axis != 1) return cudaErrorInvalidValue;
-    if (layout == LAYOUT_SOA) return axis == 0 ? walk_launch<2, LAYOUT_SOA, 0>(L) : walk_launch<2, LAYOUT_SOA, 1>(L);
-    return axis == 0 ? walk_launch<2, LAYOUT_AOS, 0>(L) : walk_launch<2, LAYOUT_AOS, 1>(L);
+    return layout == LAYOUT_SOA ? force_walk_run<2, LAYOUT_SOA>(a, grid, s) : force_walk_run<2, LAYOUT_AOS>(a, grid, s);
 }
-int force_walk_occ_f32_2d(int layout, int axis)
+int force_walk_occ_f32_2d(int layout)
 {
-    if (layout == LAYOUT_SOA) return axis == 0 ? walk_occ<2, LAYOUT_SOA, 0>() : walk_occ<2, LAYOUT_SOA, 1>();
-    return axis == 0 ? walk_occ<2, LAYOUT_AOS, 0>() : walk_occ<2, LAYOUT_AOS, 1>();
+    return layout == LAYOUT_SOA ? force_walk_occupancy<2, LAYOUT_SOA>() : force_walk_occupancy<2, LAYOUT_AOS>();
+}
+
+cudaError_t walk2d_launch_f32(int scheme, int layout, const WalkStep& a, int grid, cudaStream_t s)
+{
+    if (scheme == SCHEME_MUSCL)
+        return layout == LAYOUT_SOA ? walk2d_run<SCHEME_MUSCL, LAYOUT_SOA>(a, grid, s)
+                                    : walk2d_run<SCHEME_MUSCL, LAYOUT_AOS>(a, grid, s);
+    return layout == LAYOUT_SOA ? walk2d_run<SCHEME_RUSANOV1, LAYOUT_SOA>(a, grid, s)
+                                : walk2d_run<SCHEME_RUSANOV1, LAYOUT_AOS>(a, grid, s);
+}
+int walk2d_occ_f32(int scheme, int layout)
+{
+    if (scheme == SCHEME_MUSCL)
+        return layout == LAYOUT_SOA ? walk2d_occupancy<SCHEME_MUSCL, LAYOUT_SOA>()
+                                    : walk2d_occupancy<SCHEME_MUSCL, LAYOUT_AOS>();
+    return layout == LAYOUT_SOA ? walk2d_occupancy<SCHEME_RUSANOV1, LAYOUT_SOA>()
+                                : walk2d_occupancy<SCHEME_RUSANOV1, LAYOUT_AOS>();
 }
 }  // namespace ripple
