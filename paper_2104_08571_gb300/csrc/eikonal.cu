@@ -330,9 +330,9 @@ extern "C" ripple_status ripple_eikonal_solve(ripple_field S, ripple_field Tf, c
     }
     if (st != RIPPLE_OK) return st;
     Tf->cur = 0;
-    FieldCtl host{};
-    RIPPLE_CUDA(cudaMemcpyAsync(&host, Tf->ctl, sizeof(FieldCtl), cudaMemcpyDeviceToHost, s));
+    RIPPLE_CUDA(cudaMemcpyAsync(ctx->h_ctl, Tf->ctl, sizeof(FieldCtl), cudaMemcpyDeviceToHost, s));
     RIPPLE_CUDA(cudaStreamSynchronize(s));
+    const FieldCtl host = *ctx->h_ctl;
     if (stats) {
         stats->iterations = host.counters[0];
         stats->tile_visits = host.counters[1];

@@ -52,6 +52,9 @@ struct FieldCtl {
     unsigned int pad0;
     double totals[5];            // FP64 compensated totals (written by the totals kernel)
     long long counters[8];       // solver counters (eikonal iterations, visits, ...)
+    unsigned long long pmax;     // euler_prep_kernel: the largest wave-speed sum so far; zero between launches
+    unsigned int done;           // blocks of the prep or totals launch that have finished; zero between launches
+    unsigned int pad1;
     unsigned int bar[2];         // multi-step walk launches: grid barrier; zero between launches
     unsigned int work[4];        // and the next unit of each phase (phase number mod 4); zero between launches
 };

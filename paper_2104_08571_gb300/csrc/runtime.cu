@@ -248,8 +248,7 @@ ripple_status ensure_second_buffer(ripple_field f)
     void* p = nullptr;
     ripple_status st = ctx_alloc(f->ctx, f->bytes, &p);
     if (st != RIPPLE_OK) return st;
-    RIPPLE_CUDA(cudaMemsetAsync(p, 0, f->bytes, f->ctx->stream));
-    f->buf[1] = p;
+    f->buf[1] = p;  // every cell is written before it is read (Euler padding: pad_fill_nan_kernel)
     f->maps.clear();  // vector may reallocate: entries are re-encoded on demand
     return RIPPLE_OK;
 }
@@ -276,21 +275,15 @@ static ripple_status map_dev_err(unsigned err, const FieldCtl* host = nullptr)
 
 ripple_status take_device_error(ripple_field f)
 {
-    unsigned err = 0;
-    RIPPLE_CUDA(cudaMemcpyAsync(&err, &f->ctl->err, sizeof(unsigned), cudaMemcpyDeviceToHost, f->ctx->stream));
+    FieldCtl* h = f->ctx->h_ctl;
+    RIPPLE_CUDA(cudaMemcpyAsync(&h->err, &f->ctl->err, sizeof(unsigned), cudaMemcpyDeviceToHost, f->ctx->stream));
     RIPPLE_CUDA(cudaStreamSynchronize(f->ctx->stream));
+    const unsigned err = h->err;
     if (err) {
         RIPPLE_CUDA(cudaMemsetAsync(&f->ctl->err, 0, sizeof(unsigned), f->ctx->stream));
         RIPPLE_CUDA(cudaMemsetAsync(f->ctl->bar, 0, sizeof(f->ctl->bar) + sizeof(f->ctl->work), f->ctx->stream));
     }
     return map_dev_err(err);
-}
-
-static int grid_for(ripple_ctx ctx, long long work, int per_block)
-{
-    long long b = (work + per_block - 1) / per_block;
-    long long cap = (long long)ctx->sm_count * 8;
-    return (int)std::max<long long>(1, std::min(b, cap));
 }
 
 // Euler step dispatch -------------------------------------------------------
@@ -334,8 +327,10 @@ ripple_status ripple_ctx_create(int device, size_t mem_budget_bytes, ripple_ctx*
     c->device = device;
     c->budget = mem_budget_bytes;
     cudaError_t e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&c->h_ctl), sizeof(FieldCtl));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
+        if (c->h_ctl) cudaFreeHost(c->h_ctl);
         delete c;
         return cuda_fail(e, "ripple_ctx_create");
     }
@@ -353,6 +348,7 @@ ripple_status ripple_ctx_destroy(ripple_ctx ctx)
     ctx_free(ctx, ctx->staging, ctx->staging_bytes);
     ctx_free(ctx, ctx->partials, ctx->partials_bytes);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
+    cudaFreeHost(ctx->h_ctl);
     delete ctx;
     return RIPPLE_OK;
 }
@@ -497,10 +493,8 @@ ripple_status ripple_field_upload_device(ripple_field f, const void* src, ripple
 {
     if (!f || !src) return fail(RIPPLE_ERR_INVALID, "NULL argument");
     if (src_layout != RIPPLE_AOS && src_layout != RIPPLE_SOA) return fail(RIPPLE_ERR_INVALID, "bad layout");
-    const FieldGeom& g = f->geom;
-    const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-    RIPPLE_CUDA(launch_interior_copy(f->dtype, f->buf[f->cur], g, const_cast<void*>(src), src_layout, 0,
-                                     grid_for(f->ctx, total, 256), f->ctx->stream));
+    RIPPLE_CUDA(launch_interior_copy(f->dtype, f->buf[f->cur], f->geom, const_cast<void*>(src), src_layout, 0,
+                                     8 * f->ctx->sm_count, f->ctx->stream));
     f->prepared = false;
     return RIPPLE_OK;
 }
@@ -509,9 +503,7 @@ ripple_status ripple_field_download_device(ripple_field f, void* dst, ripple_lay
 {
     if (!f || !dst) return fail(RIPPLE_ERR_INVALID, "NULL argument");
     if (dst_layout != RIPPLE_AOS && dst_layout != RIPPLE_SOA) return fail(RIPPLE_ERR_INVALID, "bad layout");
-    const FieldGeom& g = f->geom;
-    const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-    RIPPLE_CUDA(launch_interior_copy(f->dtype, f->buf[f->cur], g, dst, dst_layout, 1, grid_for(f->ctx, total, 256),
+    RIPPLE_CUDA(launch_interior_copy(f->dtype, f->buf[f->cur], f->geom, dst, dst_layout, 1, 8 * f->ctx->sm_count,
                                      f->ctx->stream));
     return RIPPLE_OK;
 }
@@ -683,9 +675,7 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     if (!U->pad_nan) {
         // stencil items beyond the ghost layers then read NaN (ignored by the
         // admissibility minimum); prep below refills the current face ghosts
-        const long long cells = g.px * g.py * g.pz;
-        for (int b = 0; b < 2; ++b)
-            RIPPLE_CUDA(launch_pad_nan(U->dtype, U->buf[b], g, grid_for(ctx, cells, 256), ctx->stream));
+        RIPPLE_CUDA(launch_pad_nan(U->dtype, U->buf[0], U->buf[1], g, 8 * ctx->sm_count, ctx->stream));
         U->pad_nan = true;
         U->prepared = false;
     }
@@ -754,10 +744,8 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
                                 U->prep_dx[0] != p->dx[0] || U->prep_dx[1] != p->dx[1] ||
                                 (U->ndim == 3 && U->prep_dx[2] != p->dx[2]);
     if (params_changed) {
-        RIPPLE_CUDA(cudaMemsetAsync(U->ctl->smax, 0, sizeof(U->ctl->smax), s));
-        const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
         RIPPLE_CUDA(launch_prep(U->dtype, U->ndim, U->buf[U->cur], U->ctl, g, (int)p->bc, p->gamma, inv_dx,
-                                (int)(U->steps_total % 3), grid_for(ctx, total, 256), s));
+                                (int)(U->steps_total % 3), 8 * ctx->sm_count, s));
         U->prepared = true;
         U->prep_gamma = p->gamma;
         U->prep_bc = (int)p->bc;
@@ -835,9 +823,9 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
         ctx->partials_bytes = round_up(pbytes, 256);
     }
     RIPPLE_CUDA(launch_totals(U->dtype, U->ncomp, U->buf[U->cur], g, ctx->partials, nblocks, U->ctl, s));
-    FieldCtl host{};
-    RIPPLE_CUDA(cudaMemcpyAsync(&host, U->ctl, sizeof(FieldCtl), cudaMemcpyDeviceToHost, s));
+    RIPPLE_CUDA(cudaMemcpyAsync(ctx->h_ctl, U->ctl, sizeof(FieldCtl), cudaMemcpyDeviceToHost, s));
     RIPPLE_CUDA(cudaStreamSynchronize(s));
+    const FieldCtl host = *ctx->h_ctl;
     stats->t = nsteps > 0 ? host.t : 0.0;
     stats->dt_last = nsteps > 0 ? host.dt_last : 0.0;
     for (int m = 0; m < 5; ++m) stats->totals[m] = m < U->ncomp ? host.totals[m] : 0.0;

@@ -98,9 +98,9 @@ int force_walk_occ_f32_3d(int layout);
 cudaError_t walk2d_launch_f32(int scheme, int layout, const WalkStep& a, int grid, cudaStream_t s);
 int walk2d_occ_f32(int scheme, int layout);
 
-// Aux kernels (f32/f64 x 2D/3D), defined in aux.cu.
+// Aux kernels (f32/f64 x 2D/3D), defined in aux.cu; cap: most blocks of a launch.
 cudaError_t launch_prep(int dtype, int dim, void* buf, FieldCtl* ctl, const FieldGeom& g, int bc, double gamma,
-                        const double inv_dx[3], int slot, int grid, cudaStream_t s);
+                        const double inv_dx[3], int slot, int cap, cudaStream_t s);
 // Host-side fault injection for tests: RIPPLE_FAULT holds a comma-separated
 // list of host steps (alloc, admit, upload) that then fail as if the CUDA call
 // behind them had failed.  Nothing reaches the GPU: the failure is made on
@@ -108,12 +108,12 @@ cudaError_t launch_prep(int dtype, int dim, void* buf, FieldCtl* ctl, const Fiel
 bool fault_injected(const char* step);
 // Read and clear the timeout flag of the staged layout microbenchmark kernels.
 unsigned layout_bench_take_error(cudaStream_t s);
-// Quiet NaN in every non-interior cell of a padded buffer (pad_fill_nan_kernel).
-cudaError_t launch_pad_nan(int dtype, void* buf, const FieldGeom& g, int grid, cudaStream_t s);
+// Quiet NaN in every non-interior cell of both buffers (pad_fill_nan_kernel).
+cudaError_t launch_pad_nan(int dtype, void* b0, void* b1, const FieldGeom& g, int cap, cudaStream_t s);
 cudaError_t launch_totals(int dtype, int ncomp, const void* buf, const FieldGeom& g, double* partials, int nblocks,
                           FieldCtl* ctl, cudaStream_t s);
 cudaError_t launch_interior_copy(int dtype, void* buf, const FieldGeom& g, void* dense, int dense_layout, int dir,
-                                 int grid, cudaStream_t s);
+                                 int cap, cudaStream_t s);
 // Grouped admission (op 0: fill buffer 0 and clear the slot, op 1: boundary
 // images, wave speeds and buffer 1's padding) and download (op 2: pack) of
 // the batch runtime over n device-resident GroupItems (field.cuh).
@@ -148,6 +148,7 @@ struct ripple_ctx_s {
     size_t staging_bytes = 0;
     double* partials = nullptr;
     size_t partials_bytes = 0;
+    ripple::FieldCtl* h_ctl = nullptr;  // page-locked: a field's control block read back
     std::mutex mu;
     std::vector<ripple_field> fields;  // live fields (device error words read by ripple_ctx_sync)
     void* batch = nullptr;             // batch/serve runtime (batch.cu)
