@@ -30,7 +30,7 @@
 namespace ripple {
 
 template <typename T>
-cudaError_t launch_fim_init(const FimProblem<T>& a, int ts, int grid, cudaStream_t s);
+cudaError_t launch_fim_init(const FimProblem<T>& a, int ts, int grid, cudaStream_t s, FieldCtl* ctl, unsigned* bar);
 
 // ---------------------------------------------------------------------------
 // Kernel table (tile shapes are the autotuner's candidates).
@@ -569,8 +569,8 @@ static ripple_status admit(BatchRuntime* rt, Inst* in)
         const int grid = (int)std::min<long long>((total + 255) / 256, 4LL * rt->ctx->sm_count);
         RIPPLE_CUDA(launch_interior_copy(dt, in->sbuf, in->gs, in->buf[1], LAYOUT_SOA, 0, grid, s));
         RIPPLE_CUDA(cudaMemsetAsync(in->scratch, 0, in->scratch_bytes, s));
-        if (dt == RIPPLE_F32) RIPPLE_CUDA(launch_fim_init<float>(fim_problem<float>(in), EikTile<2>::TS, grid, s));
-        else RIPPLE_CUDA(launch_fim_init<double>(fim_problem<double>(in), EikTile<2>::TS, grid, s));
+        if (dt == RIPPLE_F32) RIPPLE_CUDA(launch_fim_init<float>(fim_problem<float>(in), EikTile<2>::TS, grid, s, nullptr, nullptr));
+        else RIPPLE_CUDA(launch_fim_init<double>(fim_problem<double>(in), EikTile<2>::TS, grid, s, nullptr, nullptr));
     }
     return RIPPLE_OK;
 }

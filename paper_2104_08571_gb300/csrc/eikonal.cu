@@ -3,10 +3,9 @@
 //
 // Design (GB300-native, single persistent cooperative launch):
 //   * the grid is cut into tiles (32 x 32 in 2D, 8 x 8 x 8 in 3D); an active
-//     tile is relaxed in shared memory with its ghost faces (cross stencil,
-//     no corners) by synchronous Jacobi sweeps of the Godunov upwind update
-//     T <- min(T, G(T)) until no cell moves by tol or more (or 2 x tile
-//     width sweeps);
+//     tile is relaxed in registers with its ghost faces (cross stencil, no
+//     corners) by sweeps of the Godunov upwind update T <- min(T, G(T)) until
+//     no cell moves by tol or more (fim_tile.cuh);
 //   * tiles are double-buffered across the two buffers of the T field: an
 //     active tile reads its interior and its neighbours' faces from the
 //     buffer each tile currently lives in and writes the other one, so reads
@@ -20,6 +19,11 @@
 //     DEV_ERR_TIMEOUT when the iteration cap is reached (DEV_ERR_BARRIER when
 //     a barrier wait runs out instead).
 // Outside-domain neighbours are +inf; sources stay at 0.
+//
+// What bounds it: the chain of sweeps.  An iteration lasts as long as its
+// longest visit (60 to 96 sweeps of about 0.15 us) plus 3 us of list, loads and
+// barrier.  Measured (tol 1e-6, two sources, whole solve, before -> now): 2048^2
+// 2250 -> 1410 us, 192^3 1900 -> 1320 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -34,12 +38,12 @@
 
 namespace ripple {
 
-constexpr int kFimCtasPerSm2D = 1;
+constexpr int kFimCtasPerSm2D = 2;
 
 // Arguments of the persistent single-problem solve beyond the problem itself.
 struct EikArgs {
     long long max_iters;
-    unsigned* bar;  // [2] grid barrier: arrivals, generation
+    unsigned* bar;  // grid barrier: arrivals (zero at launch)
     unsigned spin_limit;  // polls of a barrier wait before it gives up
     FieldCtl* ctl;
 };
@@ -50,18 +54,25 @@ struct EikScratch {
     int ntiles = 0;
 };
 
+// CTAs per SM the solve is compiled for.  2D: two, so that a thread may hold a
+// visit's whole state (the compiler's own choice, 64 registers, ran 2048^2 in
+// 1700 us, this 1415); 3D: six in FP32 (192^3: five 1345, six 1322, eight 1575 us).
 template <typename T, int DIM>
-__global__ void __launch_bounds__(EikTile<DIM>::NT) fim_kernel(const FimProblem<T> a, const EikArgs e)
+constexpr int fim_min_ctas() { return DIM == 2 ? 2 : sizeof(T) == 4 ? 6 : 3; }
+
+template <typename T, int DIM>
+__global__ void __launch_bounds__(EikTile<DIM>::NT, fim_min_ctas<T, DIM>()) fim_kernel(const FimProblem<T> a, const EikArgs e)
 {
     __shared__ FimSmem<T, DIM> sm;
     __shared__ int sflag[2];
-    __shared__ unsigned s_item;
+    __shared__ unsigned s_next[2];
     const int tid = threadIdx.x;
     if (tid == 0) sflag[0] = 0;
     __syncthreads();
 
     long long visits = 0, updates = 0;
     long long k = 0;
+    unsigned turn = 0;
     bool timed_out = false, barrier_out = false;
     for (;;) {
         // slots of iteration k - 1 are free: reset them for iteration k + 2
@@ -69,20 +80,22 @@ __global__ void __launch_bounds__(EikTile<DIM>::NT) fim_kernel(const FimProblem<
             a.count[(k + 2) % 3] = 0u;
             a.take[(k + 2) % 3] = 0u;
         }
-        // the active tiles of this iteration, handed out one at a time
+        // the active tiles of this iteration: each CTA takes the one of its own
+        // number, the rest are handed out one at a time (asked for before the
+        // visit in hand, so the answer is there after it)
+        const int* list = a.list + (size_t)(k % 3) * a.ntiles;
+        int t = __ldcg(list + blockIdx.x);  // read beside the count: the grid is no larger than the tiles
         const unsigned n = __ldcg(&a.count[k % 3]);
         const FimListBook<T> book{a, k};
-        for (;;) {
-            if (tid == 0) s_item = atomicAdd(&a.take[k % 3], 1u);
-            __syncthreads();
-            const unsigned i = s_item;
-            __syncthreads();
-            if (i >= n) break;
-            const int t = __ldcg(&a.list[(size_t)(k % 3) * a.ntiles + i]);
+        for (unsigned i = blockIdx.x; i < n;) {
+            if (n > gridDim.x && tid == 0) s_next[turn & 1u] = gridDim.x + atomicAdd(&a.take[k % 3], 1u);
             fim_visit_tile<T, DIM>(sm, a, t, k, visits, updates, book);
+            i = n > gridDim.x ? s_next[turn & 1u] : n;
+            ++turn;
+            if (i < n) t = __ldcg(list + i);
         }
 
-        if (!grid_barrier(e.bar, gridDim.x, e.spin_limit, sflag)) {
+        if (!grid_barrier(e.bar, (unsigned)(k + 1), e.spin_limit, sflag)) {
             barrier_out = true;
             break;
         }
@@ -126,19 +139,22 @@ __global__ void __launch_bounds__(EikTile<DIM>::NT) fim_kernel(const FimProblem<
     }
 }
 
-// Initialise both buffers (+inf interior, 0 at sources) and the active list
-// of iteration 0 (the tiles holding a source).
+// Initialise both buffers (+inf interior, 0 at sources) and the tiles of
+// iteration 0 (those holding a source): the first list with every list's
+// words (counts, marks, states, barrier) and the solver counters, or per-tile
+// flags in zeroed memory (the batched runtime).
 template <typename T>
-__global__ void fim_init_kernel(const FimProblem<T> a, int ts)
+__global__ void fim_init_kernel(const FimProblem<T> a, int ts, FieldCtl* ctl, unsigned* bar)
 {
     const FieldGeom& g = a.gT;
-    const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
     const T INF = inf_t(T(0));
-    for (long long lin = blockIdx.x * (long long)blockDim.x + threadIdx.x; lin < total;
-         lin += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(lin % g.n[0]);
-        const int j = (int)((lin / g.n[0]) % g.n[1]);
-        const int kk = (int)(lin / ((long long)g.n[0] * g.n[1]));
+    const unsigned nx = (unsigned)g.n[0], ny = (unsigned)g.n[1];
+    const long long rows = (long long)ny * g.n[2];
+    const unsigned long long total = (unsigned long long)nx * (unsigned long long)rows;
+    for (unsigned long long lin = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; lin < total;
+         lin += (unsigned long long)gridDim.x * blockDim.x) {
+        const unsigned r = (unsigned)(lin / nx);
+        const int i = (int)(lin - (unsigned long long)r * nx), j = (int)(r % ny), kk = (int)(r / ny);
         T v = INF;
         for (int q = 0; q < a.nsrc; ++q)
             if (a.src[q][0] == i && a.src[q][1] == j && (g.ndim == 2 || a.src[q][2] == kk)) v = T(0);
@@ -146,35 +162,48 @@ __global__ void fim_init_kernel(const FimProblem<T> a, int ts)
         a.buf[0][id] = v;
         a.buf[1][id] = v;
     }
+    auto tile_of = [&](int q) {
+        const int bx = a.src[q][0] / ts, by = a.src[q][1] / ts, bz = g.ndim == 3 ? a.src[q][2] / ts : 0;
+        return (bz * a.nty + by) * a.ntx + bx;
+    };
+    if (a.list) {
+        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < a.ntiles; t += gridDim.x * blockDim.x) {
+            unsigned m = 0u;
+            for (int q = 0; q < a.nsrc; ++q)
+                if (tile_of(q) == t) m = 1u;  // queued for iteration 0
+            a.mark[t] = m;
+            a.state[t] = 0u;
+        }
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        // the tiles holding a source are active in iteration 0 (per-tile flags,
-        // or the first list with each tile marked as queued for iteration 0)
         unsigned n = 0;
         for (int q = 0; q < a.nsrc; ++q) {
-            const int bx = a.src[q][0] / ts, by = a.src[q][1] / ts, bz = g.ndim == 3 ? a.src[q][2] / ts : 0;
-            const int t = (bz * a.nty + by) * a.ntx + bx;
-            if (a.list) {
-                if (a.mark[t] == 0u) {
-                    a.mark[t] = 1u;
-                    a.list[n++] = t;
-                }
-            } else if (a.act[t] == 0u) {
-                a.act[t] = 1u;
-                ++n;
-            }
+            const int t = tile_of(q);
+            bool seen = false;
+            for (int p = 0; p < q; ++p) seen |= tile_of(p) == t;
+            if (seen) continue;
+            if (a.list) a.list[n] = t;
+            else a.act[t] = 1u;
+            ++n;
         }
         a.count[0] = n;
+        if (a.list) {
+            a.count[1] = a.count[2] = 0u;
+            a.take[0] = a.take[1] = a.take[2] = 0u;
+            *bar = 0u;
+            for (int c = 0; c < 8; ++c) ctl->counters[c] = 0;
+        }
     }
 }
 
 template <typename T>
-cudaError_t launch_fim_init(const FimProblem<T>& a, int ts, int grid, cudaStream_t s)
+cudaError_t launch_fim_init(const FimProblem<T>& a, int ts, int grid, cudaStream_t s, FieldCtl* ctl, unsigned* bar)
 {
-    fim_init_kernel<T><<<grid, 256, 0, s>>>(a, ts);
+    fim_init_kernel<T><<<grid, 256, 0, s>>>(a, ts, ctl, bar);
     return cudaGetLastError();
 }
-template cudaError_t launch_fim_init<float>(const FimProblem<float>&, int, int, cudaStream_t);
-template cudaError_t launch_fim_init<double>(const FimProblem<double>&, int, int, cudaStream_t);
+template cudaError_t launch_fim_init<float>(const FimProblem<float>&, int, int, cudaStream_t, FieldCtl*, unsigned*);
+template cudaError_t launch_fim_init<double>(const FimProblem<double>&, int, int, cudaStream_t, FieldCtl*, unsigned*);
 
 void eik_scratch_free_impl(ripple_field f)
 {
@@ -216,7 +245,7 @@ void eik_scratch_free(ripple_field f) { eik_scratch_free_impl(f); }
 namespace ripple {
 size_t fim_list_scratch_bytes(int ntiles)
 {
-    // count[3] + barrier[2] + take[3] u32 (64 bytes), list[3][ntiles] i32,
+    // count[3] + barrier + take[3] u32 (64 bytes), list[3][ntiles] i32,
     // state[ntiles] u32, mark[ntiles] u32
     return (size_t)ntiles * 5 * 4 + 64;
 }
@@ -225,7 +254,6 @@ template <typename T, int DIM>
 ripple_status fim_solve_lists(FimProblem<T> a, void* scratch, FieldCtl* ctl, long long max_iters, int sm_count,
                               cudaStream_t s)
 {
-    constexpr int ts = EikTile<DIM>::TS;
     char* base = static_cast<char*>(scratch);
     a.count = reinterpret_cast<unsigned*>(base);
     a.take = reinterpret_cast<unsigned*>(base + 32);
@@ -239,23 +267,23 @@ ripple_status fim_solve_lists(FimProblem<T> a, void* scratch, FieldCtl* ctl, lon
     e.bar = reinterpret_cast<unsigned*>(base + 16);
     e.spin_limit = grid_spin_limit();
     e.ctl = ctl;
-    RIPPLE_CUDA(cudaMemsetAsync(scratch, 0, fim_list_scratch_bytes(a.ntiles), s));
-    RIPPLE_CUDA(cudaMemsetAsync(ctl->counters, 0, sizeof(ctl->counters), s));
     auto kern = fim_kernel<T, DIM>;
-    int per_sm = 0;
-    RIPPLE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, EikTile<DIM>::NT, 0));
+    static const int resident = [&] {  // CTAs per SM, 0 on error
+        int c = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, EikTile<DIM>::NT, 0) == cudaSuccess ? c : 0;
+    }();
+    int per_sm = resident;
     if (per_sm < 1) return fail(RIPPLE_ERR_INTERNAL, "FIM kernel cannot be resident");
-    // 2D solves keep a few hundred tiles active per iteration and a visit is a
-    // latency-bound chain of barrier-separated sweeps: one CTA per SM gives each
-    // visit the SM's whole issue rate (measured at 2048^2: 3.6 ms against 4.6 ms
-    // with four CTAs per SM); 3D solves have thousands of active tiles per
-    // iteration and want every resident CTA (192^3: 2.2 ms against 4.2 ms)
+    // 2D solves keep 100 to 300 tiles active per iteration, and an iteration
+    // lasts as long as its longest visit: two CTAs per SM give most visits
+    // their own issue slots (2048^2: one 1790, two 1509, four 1614 us; 1000 x 700:
+    // 622, 648, 746); 3D solves have a thousand and want every resident CTA
     if (DIM == 2) per_sm = std::min(per_sm, kFimCtasPerSm2D);
     int grid = std::min(per_sm * sm_count, a.ntiles);
     grid = std::max(grid, 1);
     const long long total = (long long)a.gT.n[0] * a.gT.n[1] * a.gT.n[2];
     const int igrid = (int)std::min<long long>((total + 255) / 256, 8LL * sm_count);
-    RIPPLE_CUDA(launch_fim_init<T>(a, ts, igrid, s));
+    RIPPLE_CUDA(launch_fim_init<T>(a, EikTile<DIM>::TS, igrid, s, ctl, e.bar));
     void* args[] = {&a, &e};
     RIPPLE_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(EikTile<DIM>::NT), args, 0, s));
     return RIPPLE_OK;
@@ -278,7 +306,6 @@ extern "C" ripple_status ripple_eikonal_solve(ripple_field S, ripple_field Tf, c
     if (nsrc < 1 || nsrc > kMaxSources) return fail(RIPPLE_ERR_INVALID, "need 1..16 sources");
     if (!(p->h > 0.0) || !(p->tol > 0.0)) return fail(RIPPLE_ERR_INVALID, "need h > 0 and tol > 0");
     const int ndim = Tf->ndim;
-    const int ts = ndim == 2 ? EikTile<2>::TS : EikTile<3>::TS;
     int ntx, nty, ntz, ntiles;
     int srcc[kMaxSources][3];
     ripple_status st = fim_describe(S, Tf, src, nsrc, p->h, p->tol, &ntx, &nty, &ntz, &ntiles, srcc);

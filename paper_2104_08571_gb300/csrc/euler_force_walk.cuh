@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_force_walk_kernel(co
             begin();
         }
         if constexpr (DIM == 3) {
-            if (!walk_barrier(ctl, ++phase, a.spin_limit, sflag)) break;
+            if (!grid_barrier(&ctl->bar[0], ++phase, a.spin_limit, sflag)) break;
             const int zper = a.zstrips * a.g.n[1];
             ForceWalk<DIM, LAYOUT, DIM - 1, false, true> wz;
             for (WalkUnits zt(ctl, phase, zper * a.zsegs, lane, warp); zt.any(); zt.advance()) {
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_force_walk_kernel(co
             }
         }
         walk_reduce(ctl, (rs + 1) % 3, smax, red);
-        if (s + 1 < a.K && !walk_barrier(ctl, ++phase, a.spin_limit, sflag)) break;
+        if (s + 1 < a.K && !grid_barrier(&ctl->bar[0], ++phase, a.spin_limit, sflag)) break;
     }
     if (sflag[0]) {
         if (tid == 0) atomicOr(&ctl->err, DEV_ERR_TIMEOUT);

@@ -31,6 +31,7 @@
 #include <cstdint>
 
 #include "batch_kernels.cuh"
+#include "grid_sync.cuh"
 
 namespace ripple {
 
@@ -58,31 +59,6 @@ __device__ __forceinline__ void solo_load(const T* __restrict__ in, const FieldG
     const long long base = geom_cell(g, x, y, 0) * g.cell_stride;
 #pragma unroll
     for (int m = 0; m < 4; ++m) q[m] = ldcg_t(in + base + (long long)m * g.comp_stride);
-}
-
-// Arrive at barrier number b (1, 2, ...) of the launch and wait until every
-// CTA has arrived.  Returns false if the wait ran out (bounded polls).  Thread
-// 0 arrives after its own earlier writes (release) and the other threads'
-// writes (the CTA barrier before it).
-__device__ __forceinline__ bool solo_barrier(unsigned* count, unsigned b, unsigned spin_limit, int* sflag)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
-        const unsigned target = b * gridDim.x;
-        uint32_t i = 0;
-        for (;;) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-            if (v >= target) break;
-            if (++i > spin_limit) {
-                sflag[0] = 1;
-                break;
-            }
-        }
-    }
-    __syncthreads();
-    return sflag[0] == 0;
 }
 
 // Registers of a warp's current unit: the rows below, at, above and two above
@@ -220,7 +196,7 @@ __global__ void __launch_bounds__(kSoloThreads) solo_euler2d_kernel(const SoloEu
             for (int i = 1; i < wpc; ++i) m = max(m, s_max[i]);
             atomic_max_pos_double(&ctl->smax[(rs + 1) % 3], (double)m);
         }
-        if (k + 1 < a.K && !solo_barrier(a.bar, (unsigned)(k + 1), a.spin_limit, sflag)) {
+        if (k + 1 < a.K && !grid_barrier(a.bar, (unsigned)(k + 1), a.spin_limit, sflag)) {
             if (threadIdx.x == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
             return;
         }

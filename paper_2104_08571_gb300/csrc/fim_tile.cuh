@@ -4,11 +4,25 @@
 //
 // Which tiles iteration k visits, and which buffer each tile lives in, is the
 // business of a bookkeeping policy (per-tile flags or lists of active tiles,
-// below).  An active tile is staged in shared memory (its interior from the buffer it
-// lives in, the faces of its neighbours from theirs), relaxed by synchronous
-// Jacobi sweeps of T <- min(T, G(T)) until no cell moves by tol, and written to
-// its other buffer; a tile that did not converge stays active and a boundary
-// layer that moved by tol or more activates the neighbour across that face.
+// below).  An active tile is read into registers (its interior from the buffer
+// it lives in, the faces of its neighbours from theirs), relaxed by sweeps of
+// T <- min(T, G(T)) until no cell moves by tol, and written to its other
+// buffer; a tile that did not converge stays active and a boundary layer that
+// moved by tol or more activates the neighbour across that face.
+//
+// A solve follows one chain: a front crosses a tile one cell per sweep, and
+// iterations follow each other, so what counts is the latency of a sweep and
+// of what surrounds it, not the number of updates.  Hence:
+//   * four cells per thread stay in registers for the whole visit; neighbours
+//     in the warp come by shuffles, those in the thread from registers, and
+//     only the layers between two warps pass through shared memory;
+//   * kFimInner sweeps run between two exchanges of those layers, so a CTA
+//     barrier (which also decides convergence) is paid once per exchange;
+//   * everything a visit reads is requested at once: both buffers' values with
+//     the words that say which one counts, so the visit starts after one trip
+//     to L2 instead of three;
+//   * the update has no branches.
+// (Before: cells in shared memory, five loads and a barrier per sweep.)
 #pragma once
 #include <cstdint>
 
@@ -39,53 +53,55 @@ __device__ __forceinline__ float fim_sqrt(float x)
 }
 __device__ __forceinline__ double fim_sqrt(double x) { return sqrt(x); }
 
+__device__ __forceinline__ float fim_min3(float a, float b, float c)
+{
+    float r;  // one instruction on sm_100 and later
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ double fim_min3(double a, double b, double c) { return fmin(fmin(a, b), c); }
+
 // Godunov upwind local solver: a[d] = smaller neighbour value along axis d,
-// f = s * h.  2D: one-sided if |a0 - a1| >= f, else the two-sided root.
-// 3D: sorted a1 <= a2 <= a3, add terms while the candidate exceeds the next.
+// f = s * h.  Written for the distance u above the smallest neighbour, without
+// branches:
+//   2D: u is the larger root of u^2 + (u - d)^2 = f^2, d the distance between
+//       the two; at d = f the root is f, the one-sided value, so clamping d at
+//       f covers both cases;
+//   3D (sorted, p and q the distances to the second and third): the 2D value
+//       of the first two, or, if that exceeds q, the larger root of u^2 + (u -
+//       p)^2 + (u - q)^2 = f^2.
+// Only differences enter the roots, so nothing of size T^2 cancels.  Infinite
+// neighbours give infinite or NaN distances, which the minimum or the
+// comparison passes over; f = inf gives inf (a cell that keeps its value).
 template <typename T, int DIM>
 __device__ __forceinline__ T godunov(T a0, T a1, T a2, T f)
 {
+    const T ff = f * f;
     if (DIM == 2) {
-        const T lo = fmin(a0, a1);
-        const T d = a0 - a1;
-        if (!(fabs(d) < f)) return lo + f;
-        return T(0.5) * (a0 + a1 + fim_sqrt(T(2) * f * f - d * d));
+        const T lo = fmin(a0, a1), d = fmin(fmax(a0, a1) - lo, f);
+        return lo + T(0.5) * (d + fim_sqrt(T(2) * ff - d * d));
     } else {
-        // sort ascending
-        T x = fmin(a0, a1), y = fmax(a0, a1);
-        T z = fmax(y, a2);
-        y = fmin(y, a2);
-        const T x2 = fmin(x, y);
-        y = fmax(x, y);
-        x = x2;
-        T t = x + f;
-        if (!(t > y)) return t;
-        const T d = x - y;
-        t = T(0.5) * (x + y + fim_sqrt(T(2) * f * f - d * d));
-        if (!(t > z)) return t;
-        // three terms: 3T^2 - 2 S T + (Q - f^2) = 0.  Its discriminant
-        // S^2 - 3 (Q - f^2) equals 3 f^2 - sum of squared pairwise differences;
-        // the second form has no cancellation between terms of size T^2
-        // (which in FP32 would swamp f^2 on fine grids).
-        const T dxy = x - y, dxz = x - z, dyz = y - z;
-        const T disc = fmax(T(3) * f * f - (dxy * dxy + dxz * dxz + dyz * dyz), T(0));
-        return (x + y + z + fim_sqrt(disc)) * (T(1) / T(3));
+        const T lo = fmin(a0, a1), hi = fmax(a0, a1);
+        const T x = fmin(lo, a2), z = fmax(hi, a2), y = fmax(lo, fmin(hi, a2));
+        const T p = y - x, q = z - x, d = fmin(p, f);
+        const T u2 = T(0.5) * (d + fim_sqrt(T(2) * ff - d * d));
+        const T disc = fmax(T(3) * ff - T(2) * (p * (p - q) + q * q), T(0));
+        const T u3 = (p + q + fim_sqrt(disc)) * (T(1) / T(3));
+        return x + (u2 > q ? u3 : u2);
     }
 }
 
 template <int DIM>
 struct EikTile {
     static constexpr int TS = DIM == 2 ? 32 : 8;
-    // threads per tile: a tile visit is a chain of Jacobi sweeps, so more threads
-    // per 32 x 32 tile (two cells each) shorten every sweep; 8^3 tiles keep 256
-    static constexpr int NT = DIM == 2 ? 512 : 256;
     static constexpr int CELLS = DIM == 2 ? TS * TS : TS * TS * TS;
-    static constexpr int CPT = CELLS / NT;  // cells per thread
-    static constexpr int P = TS + 2;        // padded tile side
-    static constexpr int PCELLS = DIM == 2 ? P * P : P * P * P;
-    static constexpr int MAX_SWEEPS = 2 * TS * (DIM == 3 ? 3 : 1);
+    static constexpr int CPT = 4;           // cells per thread: rows (2D) or z layers (3D)
+    static constexpr int NT = CELLS / CPT;  // threads per tile: 8 warps (2D), 4 warps (3D)
+    // a visit ends unconverged after this many: visits are cheapest when almost
+    // all of them converge (2048^2: 1509 us at 96, 1700 at 64, 2826 at 48)
+    static constexpr int MAX_SWEEPS = DIM == 2 ? 96 : 64;
 };
-
+constexpr int kFimInner = 2;  // sweeps between two exchanges (2048^2: 1 1674, 2 1509, 4 1540 us)
 
 // Per-problem state of the FIM iteration.  Two bookkeeping schemes use it:
 //   flags (the batched runtime): act[3][ntiles] active flags and cur[2][ntiles]
@@ -121,15 +137,18 @@ struct FimFlagBook {
     const FimProblem<T>& a;
     long long k;
     __device__ unsigned char buf_of(int t) const { return __ldcg(&a.cur[(size_t)(k % 2) * a.ntiles + t]); }
-    __device__ bool begin(int t, unsigned char& cb) const
+    __device__ bool active(int t) const
     {
         const unsigned is_active = __ldcg(&a.act[(size_t)(k % 3) * a.ntiles + t]);
-        cb = buf_of(t);
         if (threadIdx.x == 0) {
             a.act[(size_t)((k + 2) % 3) * a.ntiles + t] = 0u;
-            a.cur[(size_t)((k + 1) % 2) * a.ntiles + t] = is_active ? (unsigned char)(1 - cb) : cb;
+            if (!is_active) a.cur[(size_t)((k + 1) % 2) * a.ntiles + t] = buf_of(t);
         }
         return is_active != 0u;
+    }
+    __device__ void begin(int t, unsigned char cb) const
+    {
+        if (threadIdx.x == 0) a.cur[(size_t)((k + 1) % 2) * a.ntiles + t] = (unsigned char)(1 - cb);
     }
     __device__ void activate(int nb) const
     {
@@ -151,12 +170,11 @@ struct FimListBook {
         const unsigned char b = (unsigned char)(w & 1u);
         return (w >> 1) == (unsigned)(k + 1) ? (unsigned char)(b ^ 1u) : b;
     }
-    __device__ bool begin(int t, unsigned char& cb) const
+    __device__ bool active(int) const { return true; }
+    // (a thread that reads the word after this still sees the old buffer)
+    __device__ void begin(int t, unsigned char cb) const
     {
-        cb = buf_of(t);
-        __syncthreads();  // every thread has its buffer index before the word changes
         if (threadIdx.x == 0) a.state[t] = ((unsigned)(k + 1) << 1) | (unsigned)(1 - cb);
-        return true;
     }
     __device__ void activate(int nb) const
     {
@@ -168,163 +186,222 @@ struct FimListBook {
     }
 };
 
+// Layers that pass between the warps of a tile, double-buffered by exchange.
 template <typename T, int DIM>
-struct FimSmem {
-    T sa[EikTile<DIM>::PCELLS];
-    T sb[EikTile<DIM>::PCELLS];
+struct FimSmem;
+template <typename T>
+struct FimSmem<T, 2> {
+    T top[2][8][32], bot[2][8][32];  // first and last row of each warp
+    unsigned side_mask;
+};
+template <typename T>
+struct FimSmem<T, 3> {
+    T zl[2][4][32];    // each warp's layer at the tile's middle in z
+    T yl[2][4][4][8];  // each warp's rows at the tile's middle in y, [z][x]
     unsigned side_mask;
 };
 
 // Visit tile t of problem `a` in iteration k (all threads of the CTA call it)
 // with the bookkeeping `book` (FimFlagBook or FimListBook).  Adds one tile
 // visit and the Godunov updates performed to the counters.
+// 2D: warp w holds rows 4w .. 4w + 3, lane x column x.  3D: warp w holds rows
+// y = 4 (w & 1) + lane / 8, columns x = lane % 8, layers z = 4 (w >> 1) + 0 .. 3.
 template <typename T, int DIM, class Book>
 __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimProblem<T>& a, int t, long long k,
                                                long long& visits, long long& updates, const Book& book)
 {
     using C = EikTile<DIM>;
-    constexpr int TS = C::TS, P = C::P, CPT = C::CPT;
-    const int tid = threadIdx.x;
+    constexpr int TS = C::TS, CPT = C::CPT, W = TS;  // W: lanes of one row
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const T INF = inf_t(T(0));
     const T tol = (T)a.tol;
     const FieldGeom& gT = a.gT;
     const FieldGeom& gS = a.gS;
-    T* sa = sm.sa;
-    T* sb = sm.sb;
 
-    auto cell_xyz = [&](int c, int& x, int& y, int& z) {  // thread cell c: linear cell tid + c * NT
-        const int lin = tid + c * C::NT;
-        x = lin % TS;
-        y = (lin / TS) % TS;
-        z = DIM == 3 ? lin / (TS * TS) : 0;
-    };
-    auto pidx = [&](int x, int y, int z) -> int {  // padded smem index, x,y,z in [-1, TS]
-        return DIM == 2 ? (y + 1) * P + (x + 1) : ((z + 1) * P + (y + 1)) * P + (x + 1);
-    };
-
-    unsigned char cb;
-    if (!book.begin(t, cb)) return;
+    if (!book.active(t)) return;
     ++visits;
     const int bx = t % a.ntx, by = (t / a.ntx) % a.nty, bz = DIM == 3 ? t / (a.ntx * a.nty) : 0;
-    const int x0 = bx * TS, y0 = by * TS, z0 = bz * TS;
-    const T* src_buf = a.buf[cb];
-    T* dst_buf = a.buf[1 - cb];
+    const int lx = DIM == 2 ? lane : lane & 7;
+    const int ly = DIM == 2 ? CPT * w : 4 * (w & 1) + (lane >> 3);
+    const int lz = DIM == 2 ? 0 : CPT * (w >> 1);
+    const int gx = bx * TS + lx, gy = by * TS + ly, gz = bz * TS + lz;
+    const long long cstep = DIM == 2 ? gT.px : gT.px * gT.py;  // from one of the thread's cells to the next
+    const long long id0 = geom_cell(gT, gx, gy, gz);
+    const long long is0 = geom_cell(gS, gx, gy, gz) * gS.cell_stride;
+    const long long sstep = (DIM == 2 ? gS.px : gS.px * gS.py) * gS.cell_stride;
+    const int nrun = DIM == 2 ? gT.n[1] - gy : gT.n[2] - gz;  // cells of the run inside the grid
+    const bool col = gx < gT.n[0] && (DIM == 2 || gy < gT.n[1]);
+    const T* b0 = a.buf[0];
+    const T* b1 = a.buf[1];
 
-    // ---- stage the tile: interior from this tile's buffer, faces from the neighbours' ----
-    for (int i = tid; i < C::PCELLS; i += C::NT) { sa[i] = INF; sb[i] = INF; }
-    __syncthreads();
-    T init[CPT], fh[CPT];
-    bool fixed[CPT];
-    int cid[CPT];  // padded shared-memory index of each of this thread's cells
+    // ---- everything the visit reads, in one go ----
+    // neighbours outside the warps: x ghosts of the edge columns (one per cell),
+    // the row or layer before the first cell of the run and after the last (the
+    // edge warps only), 3D: y ghosts of the edge rows (one per cell)
+    const bool xlo = lx == 0, xhi = lx == TS - 1;
+    const int tx_nb = xlo ? (bx > 0 ? t - 1 : -1) : xhi ? (bx + 1 < a.ntx ? t + 1 : -1) : -1;
+    const int run_tiles = DIM == 2 ? a.ntx : a.ntx * a.nty;  // tile distance along the run
+    const bool r_lo = DIM == 2 ? w == 0 : w < 2, r_hi = DIM == 2 ? w == 7 : w >= 2;
+    const int tr_nb = r_lo ? ((DIM == 2 ? by : bz) > 0 ? t - run_tiles : -1)
+                      : r_hi ? ((DIM == 2 ? by + 1 < a.nty : bz + 1 < a.ntz) ? t + run_tiles : -1)
+                             : -1;
+    const bool ylo = DIM == 3 && (w & 1) == 0 && lane < 8, yhi = DIM == 3 && (w & 1) == 1 && lane >= 24;
+    const int ty_nb = ylo ? (by > 0 ? t - a.ntx : -1) : yhi ? (by + 1 < a.nty ? t + a.ntx : -1) : -1;
+    T v[CPT], v1[CPT], f[CPT], xg[CPT], xg1[CPT], yg[CPT], yg1[CPT];
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
-        int x, y, z;
-        cell_xyz(c, x, y, z);
-        const int gx = x0 + x, gy = y0 + y, gz = z0 + z;
-        const bool valid = gx < gT.n[0] && gy < gT.n[1] && gz < gT.n[2];
-        T v = INF;
-        bool src = false;
-        fh[c] = T(0);
-        cid[c] = pidx(x, y, z);
-        if (valid) {
-            v = ldcg_t(&src_buf[geom_cell(gT, gx, gy, gz)]);
-            fh[c] = a.slow[geom_cell(gS, gx, gy, gz) * gS.cell_stride] * (T)a.h;
-            for (int q = 0; q < a.nsrc; ++q)
-                src |= (a.src[q][0] == gx) & (a.src[q][1] == gy) & (DIM == 2 || a.src[q][2] == gz);
+        const bool in = col && c < nrun;
+        const long long id = id0 + c * cstep;
+        v[c] = v1[c] = xg[c] = xg1[c] = yg[c] = yg1[c] = f[c] = INF;
+        if (in) {
+            v[c] = ldcg_t(b0 + id);
+            v1[c] = ldcg_t(b1 + id);
+            f[c] = a.slow[is0 + c * sstep];
         }
-        init[c] = v;
-        fixed[c] = !valid || src;
-        sa[pidx(x, y, z)] = v;
-        sb[pidx(x, y, z)] = v;
-    }
-    // ghost faces: 2*DIM faces of TS^(DIM-1) cells
-    constexpr int FACE = DIM == 2 ? TS : TS * TS;
-    for (int i = tid; i < 2 * DIM * FACE; i += C::NT) {
-        const int face = i / FACE, r = i % FACE;
-        const int axis = face >> 1, side = face & 1;
-        int u = r % TS, w = r / TS;  // in-face coordinates
-        int lx, ly, lz;
-        if (axis == 0) { lx = side ? TS : -1; ly = u; lz = w; }
-        else if (axis == 1) { lx = u; ly = side ? TS : -1; lz = w; }
-        else { lx = u; ly = w; lz = side ? TS : -1; }
-        if (DIM == 2) lz = 0;
-        const int gx = x0 + lx, gy = y0 + ly, gz = z0 + lz;
-        T v = INF;
-        if (gx >= 0 && gy >= 0 && gz >= 0 && gx < gT.n[0] && gy < gT.n[1] && gz < gT.n[2]) {
-            const int nbx = gx / TS, nby = gy / TS, nbz = gz / TS;
-            const int nb = DIM == 2 ? nby * a.ntx + nbx : (nbz * a.nty + nby) * a.ntx + nbx;
-            v = ldcg_t(&a.buf[book.buf_of(nb)][geom_cell(gT, gx, gy, gz)]);
+        if (in && tx_nb >= 0) {
+            xg[c] = ldcg_t(b0 + id + (xlo ? -1 : 1));
+            xg1[c] = ldcg_t(b1 + id + (xlo ? -1 : 1));
         }
-        sa[pidx(lx, ly, lz)] = v;
-        sb[pidx(lx, ly, lz)] = v;
+        if (DIM == 3 && in && ty_nb >= 0) {
+            yg[c] = ldcg_t(b0 + id + (ylo ? -gT.px : gT.px));
+            yg1[c] = ldcg_t(b1 + id + (ylo ? -gT.px : gT.px));
+        }
     }
-    __syncthreads();
-
-    // ---- Jacobi sweeps in shared memory ----
-    T* A = sa;
-    T* B = sb;
-    bool converged = false;
-    int sweeps = 0;
-    for (; sweeps < C::MAX_SWEEPS; ++sweeps) {
-        bool moved = false;
+    T rg = INF, rg1 = INF;
+    if (col && tr_nb >= 0) {
+        const long long id = r_lo ? id0 - cstep : id0 + CPT * cstep;
+        rg = ldcg_t(b0 + id);
+        rg1 = ldcg_t(b1 + id);
+    }
+    const unsigned char cb = book.buf_of(t);
+    const bool xb = tx_nb >= 0 && book.buf_of(tx_nb) != 0, rb = tr_nb >= 0 && book.buf_of(tr_nb) != 0;
+    const bool yb = DIM == 3 && ty_nb >= 0 && book.buf_of(ty_nb) != 0;
+    book.begin(t, cb);
+    T init[CPT];
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) {
-            if (fixed[c]) continue;
-            const int id = cid[c];
-            const T old = A[id];
-            const T ax = fmin(A[id - 1], A[id + 1]);
-            const T ay = fmin(A[id - P], A[id + P]);
-            const T az = DIM == 3 ? fmin(A[id - P * P], A[id + P * P]) : INF;
-            const T g = godunov<T, DIM>(ax, ay, az, fh[c]);
-            const T nv = fmin(old, g);
-            B[id] = nv;
-            moved |= (old - nv) >= tol;
+    for (int c = 0; c < CPT; ++c) {
+        if (cb) v[c] = v1[c];
+        if (xb) xg[c] = xg1[c];
+        if (yb) yg[c] = yg1[c];
+        init[c] = v[c];
+        f[c] = f[c] * (T)a.h;  // outside the grid: infinite, so the cell keeps its (infinite) value
+    }
+    if (rb) rg = rg1;
+    // sources keep their value
+    for (int q = 0; q < a.nsrc; ++q) {
+        if (a.src[q][0] != gx || (DIM == 3 && a.src[q][1] != gy)) continue;
+        const int c = DIM == 2 ? a.src[q][1] - gy : a.src[q][2] - gz;
+#pragma unroll
+        for (int e = 0; e < CPT; ++e)
+            if (c == e) f[e] = INF;
+    }
+
+    // ---- sweeps ----
+    bool converged = false, moved = true;
+    int sweeps = 0, par = 0;
+    T lo = rg, hi = rg;  // the neighbours of the run's first and last cell
+    for (;;) {
+        // exchange the layers between warps; the barrier also tells whether any
+        // cell has moved since the last one
+        if (DIM == 2) {
+            if constexpr (DIM == 2) {
+                sm.top[par][w][lane] = v[0];
+                sm.bot[par][w][lane] = v[CPT - 1];
+            }
+        } else {
+            if constexpr (DIM == 3) {
+                sm.zl[par][w][lane] = r_lo ? v[CPT - 1] : v[0];
+                if ((w & 1) == 0 ? lane >= 24 : lane < 8) {
+#pragma unroll
+                    for (int c = 0; c < CPT; ++c) sm.yl[par][w][c][lx] = v[c];
+                }
+            }
         }
-        const int any = __syncthreads_or(moved ? 1 : 0);
-        T* tmp = A;
-        A = B;
-        B = tmp;
-        if (!any) {
+        if (!__syncthreads_or(moved ? 1 : 0)) {
             converged = true;
-            ++sweeps;
             break;
         }
+        if (sweeps >= C::MAX_SWEEPS) break;
+        if constexpr (DIM == 2) {
+            if (w > 0) lo = sm.bot[par][w - 1][lane];
+            if (w < 7) hi = sm.top[par][w + 1][lane];
+        } else {
+            if (r_lo) hi = sm.zl[par][w ^ 2][lane];
+            else lo = sm.zl[par][w ^ 2][lane];
+            if ((w & 1) == 0 ? lane >= 24 : lane < 8) {
+#pragma unroll
+                for (int c = 0; c < CPT; ++c) yg[c] = sm.yl[par][w ^ 1][c][lx];
+            }
+        }
+        moved = false;
+#pragma unroll
+        for (int s = 0; s < kFimInner; ++s) {
+            T nv[CPT];
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) {
+                // at the warp's edges the shuffle returns the cell's own value, which
+                // changes nothing (a candidate above the cell's value is dropped),
+                // and the ghost is the third operand (infinite elsewhere)
+                const T l = __shfl_up_sync(0xffffffffu, v[c], 1, W), r = __shfl_down_sync(0xffffffffu, v[c], 1, W);
+                const T below = c == 0 ? lo : v[c == 0 ? 0 : c - 1], above = c == CPT - 1 ? hi : v[c == CPT - 1 ? c : c + 1];
+                T g;
+                if constexpr (DIM == 2) {
+                    g = godunov<T, 2>(fim_min3(l, r, xg[c]), fmin(below, above), INF, f[c]);
+                } else {
+                    const T u = __shfl_up_sync(0xffffffffu, v[c], 8), d = __shfl_down_sync(0xffffffffu, v[c], 8);
+                    g = godunov<T, 3>(fim_min3(l, r, xg[c]), fim_min3(u, d, yg[c]), fmin(below, above), f[c]);
+                }
+                nv[c] = fmin(v[c], g);
+                moved |= v[c] - nv[c] >= tol;
+            }
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) v[c] = nv[c];
+        }
+        sweeps += kFimInner;
+        par ^= 1;
     }
     updates += (long long)sweeps * C::CELLS;
 
     // ---- write back; boundary-layer changes activate neighbours ----
     if (tid == 0) sm.side_mask = 0u;
     __syncthreads();
-    unsigned mask = 0u;
+    T* out = a.buf[1 - cb];
+    bool any = false, first = false, last = false;
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
-        int x, y, z;
-        cell_xyz(c, x, y, z);
-        const int gx = x0 + x, gy = y0 + y, gz = z0 + z;
-        const bool valid = gx < gT.n[0] && gy < gT.n[1] && gz < gT.n[2];
-        const T v = A[pidx(x, y, z)];
-        if (valid) dst_buf[geom_cell(gT, gx, gy, gz)] = v;
-        if (valid && (init[c] - v) >= tol) {
-            if (x == 0) mask |= 1u;
-            if (x == TS - 1) mask |= 2u;
-            if (y == 0) mask |= 4u;
-            if (y == TS - 1) mask |= 8u;
-            if (DIM == 3 && z == 0) mask |= 16u;
-            if (DIM == 3 && z == TS - 1) mask |= 32u;
-        }
+        if (col && c < nrun) out[id0 + c * cstep] = v[c];
+        const bool ch = init[c] - v[c] >= tol;
+        any |= ch;
+        if (c == 0) first = ch && r_lo;
+        if (c == CPT - 1) last = ch && r_hi;
     }
-    if (mask) atomicOr(&sm.side_mask, mask);
+    const unsigned by_lane = __ballot_sync(0xffffffffu, any);
+    const bool b_first = __any_sync(0xffffffffu, first), b_last = __any_sync(0xffffffffu, last);
+    if (lane == 0) {
+        unsigned m;  // bits: x low, x high, y low, y high, z low, z high
+        if (DIM == 2) {
+            m = (by_lane & 1u) | ((by_lane >> 31) << 1) | (b_first ? 4u : 0u) | (b_last ? 8u : 0u);
+        } else {
+            m = ((by_lane & 0x01010101u) ? 1u : 0u) | ((by_lane & 0x80808080u) ? 2u : 0u) |
+                ((w & 1) == 0 && (by_lane & 0xffu) ? 4u : 0u) | ((w & 1) == 1 && (by_lane >> 24) ? 8u : 0u) |
+                (b_first ? 16u : 0u) | (b_last ? 32u : 0u);
+        }
+        if (m) atomicOr(&sm.side_mask, m);
+    }
     __syncthreads();
-    if (tid == 0) {
-        auto activate = [&](int nb) { book.activate(nb); };
-        if (!converged) activate(t);
+    if (tid <= 2 * DIM) {
+        // one thread per tile that may become active: this one, then across each side
         const unsigned m = sm.side_mask;
-        if ((m & 1u) && bx > 0) activate(t - 1);
-        if ((m & 2u) && bx + 1 < a.ntx) activate(t + 1);
-        if ((m & 4u) && by > 0) activate(t - a.ntx);
-        if ((m & 8u) && by + 1 < a.nty) activate(t + a.ntx);
-        if (DIM == 3 && (m & 16u) && bz > 0) activate(t - a.ntx * a.nty);
-        if (DIM == 3 && (m & 32u) && bz + 1 < a.ntz) activate(t + a.ntx * a.nty);
+        const int side = tid - 1, axis = side >> 1;
+        int nb = -1;
+        if (tid == 0) nb = converged ? -1 : t;
+        else if (m >> side & 1u) {
+            const int pos = axis == 0 ? bx : axis == 1 ? by : bz, cnt = axis == 0 ? a.ntx : axis == 1 ? a.nty : a.ntz;
+            const int dist = axis == 0 ? 1 : axis == 1 ? a.ntx : a.ntx * a.nty;
+            if (side & 1) nb = pos + 1 < cnt ? t + dist : -1;
+            else nb = pos > 0 ? t - dist : -1;
+        }
+        if (nb >= 0) book.activate(nb);
     }
     __syncthreads();
 }

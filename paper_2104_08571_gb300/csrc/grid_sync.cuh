@@ -1,5 +1,5 @@
 // Bounded grid-wide barrier of the persistent cooperative kernels (the FIM
-// solve and the multi-step solo Euler solver).
+// solve, the multi-step solo Euler solver and the strip walks).
 #pragma once
 #include <cstdint>
 #include <cstdlib>
@@ -21,32 +21,28 @@ inline unsigned grid_spin_limit()
     return limit;
 }
 
-// Bounded sense-reversal grid barrier over bar[0] (arrivals, reset by the
-// last arrival) and bar[1] (generation).  Every CTA of the grid calls it the
-// same number of times; sflag (shared memory) records a wait that ran out, and
-// the call returns false from then on.
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks, unsigned spin_limit, int* sflag)
+// Grid barrier number b (1, 2, ...) of a launch over an arrival counter that
+// only counts up (zero when the launch begins), with bounded polls.  Thread 0
+// arrives with a release after the CTA barrier, so the CTA's stores precede
+// it; its acquire and the second CTA barrier order the other CTAs' stores
+// before every later load of this CTA.  sflag (shared memory) records a wait
+// that ran out, and the call returns false from then on.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned b, unsigned spin_limit, int* sflag)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned* gen = bar + 1;
-        const unsigned g0 = *gen;
-        __threadfence();
-        if (atomicAdd(bar, 1u) == nblocks - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            uint32_t i = 0;
-            while (*gen == g0) {
-                if (i++ >= spin_limit) {
-                    sflag[0] = 1;
-                    break;
-                }
-                __nanosleep(32);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        const unsigned target = b * gridDim.x;
+        uint32_t i = 0;
+        for (;;) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (++i > spin_limit) {
+                sflag[0] = 1;
+                break;
             }
         }
-        __threadfence();
     }
     __syncthreads();
     return sflag[0] == 0;

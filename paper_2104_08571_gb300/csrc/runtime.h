@@ -65,8 +65,8 @@ int sweep_smem(ripple_dtype dt, int dim, int layout, int scheme, int v);
 int sweep_occ(ripple_dtype dt, int dim, int layout, int scheme, int v);
 
 // One eikonal solve by the persistent FIM kernel with lists of active tiles
-// (eikonal.cu), queued on s: zeroes `scratch` (fim_list_scratch_bytes bytes)
-// and ctl's solver counters, initialises both T buffers and the first list,
+// (eikonal.cu), queued on s: sets up `scratch` (fim_list_scratch_bytes bytes)
+// and zeroes ctl's solver counters, initialises both T buffers and the first list,
 // launches the cooperative solve; the result is in buf[0], the iterations,
 // tile visits and Godunov updates in ctl->counters[0..2], errors in ctl->err.
 template <typename T>

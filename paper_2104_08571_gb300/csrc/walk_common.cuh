@@ -11,6 +11,7 @@
 #include <cstdint>
 
 #include "euler_sweep.cuh"
+#include "grid_sync.cuh"
 #include "pair_math.cuh"
 #include "tma.cuh"
 
@@ -38,36 +39,12 @@ struct WalkStep {
     unsigned spin_limit;   // polls of a barrier wait before it gives up
 };
 
-// Grid barrier of a launch over ctl->bar[0] (arrivals, counted up over the
-// launch) with bounded polls.  Thread 0 arrives with a release after the CTA
-// barrier, so the CTA's stores precede it; its acquire and the second CTA
-// barrier order the other CTAs' stores before every later load of this CTA.
-// The last CTA to leave the kernel (walk_leave) sets both words back to zero,
-// so a launch needs no reset before it.  Returns false when a wait ran out.
-// (Every acquiring poll drops the SM's L1 lines, which a second CTA on the SM
-// would still be working on: 230 against 169 us a step for 4096^2 FORCE with
-// two CTAs of 8 warps per SM.  One CTA of 16 has no such neighbour.)
-__device__ __forceinline__ bool walk_barrier(FieldCtl* ctl, unsigned b, unsigned spin_limit, int* sflag)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar[0]) : "memory");
-        const unsigned target = b * gridDim.x;
-        uint32_t i = 0;
-        for (;;) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->bar[0]) : "memory");
-            if (v >= target) break;
-            if (++i > spin_limit) {
-                sflag[0] = 1;
-                break;
-            }
-        }
-    }
-    __syncthreads();
-    return sflag[0] == 0;
-}
-
+// The launch's grid barriers count up ctl->bar[0] (grid_sync.cuh); the last CTA
+// to leave the kernel sets the barrier's and the units' words back to zero, so
+// a launch needs no reset before it.  (Every acquiring poll drops the SM's L1
+// lines, which a second CTA on the SM would still be working on: 230 against
+// 169 us a step for 4096^2 FORCE with two CTAs of 8 warps per SM.  One CTA of
+// 16 has no such neighbour.)
 // Every CTA calls this once, after its last barrier.
 __device__ __forceinline__ void walk_leave(FieldCtl* ctl)
 {
