@@ -287,13 +287,18 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
         f[c] = f[c] * (T)a.h;  // outside the grid: infinite, so the cell keeps its (infinite) value
     }
     if (rb) rg = rg1;
-    // sources keep their value
+    // sources keep their value; in the first iteration they count as changed, so
+    // that a source on a tile's edge reaches the tile beside it even when no
+    // other cell of its tile does
     for (int q = 0; q < a.nsrc; ++q) {
         if (a.src[q][0] != gx || (DIM == 3 && a.src[q][1] != gy)) continue;
         const int c = DIM == 2 ? a.src[q][1] - gy : a.src[q][2] - gz;
 #pragma unroll
         for (int e = 0; e < CPT; ++e)
-            if (c == e) f[e] = INF;
+            if (c == e) {
+                f[e] = INF;
+                if (k == 0) init[e] = INF;
+            }
     }
 
     // ---- sweeps ----

@@ -36,7 +36,7 @@ def _solve(ctx, s, src, h, dtype, tol):
 
 CASES = [((1, 40), [(0, 39)]), ((31, 3), [(30, 2)]), ((32, 32), [(0, 0), (31, 31), (31, 0)]),
          ((33, 33), [(31, 32)]), ((64, 5), [(31, 4), (32, 4)]), ((100, 97), [(31, 32), (63, 64), (96, 0)]),
-         ((1, 1, 9), [(0, 0, 7)]), ((8, 8, 8), [(7, 7, 7), (0, 0, 0)]), ((9, 7, 17), [(8, 3, 8)]),
+         ((1, 1, 9), [(0, 0, 7)]), ((33, 33), [(32, 32)]), ((1, 1, 9), [(0, 0, 8)]), ((8, 8, 8), [(7, 7, 7), (0, 0, 0)]), ((9, 7, 17), [(8, 3, 8)]),
          ((16, 5, 12), [(7, 3, 3), (8, 4, 4)]), ((25, 30, 20), [(12, 15, 11), (0, 29, 19)])]
 
 
