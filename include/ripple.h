@@ -291,9 +291,11 @@ typedef struct {
     int64_t active_cells;     /* per-step cell budget of stepped Euler problems, chosen by least
                                  remaining work (0 = step every resident problem) */
     int staging;              /* halo staging of the Euler step: 0 = TMA tile loads by a producer warp
-                                 into a shared-memory ring; 1 = direct loads by every thread; 2 = no
-                                 tiles: warps walk 30-column x 16-row units (x faces by shuffles, the
-                                 y face carried); the results are the same bits either way */
+                                 into a shared-memory ring (FP64 steps and dependency-driven rounds;
+                                 FP32 steps launched one by one walk as with 2, which is faster); 1 =
+                                 direct loads by every thread; 2 = no tiles: warps walk strips of rows
+                                 (x faces by shuffles, the y face carried); the results are the same
+                                 bits either way */
     int async_queue;          /* 1 = dependency-driven rounds: ONE persistent launch runs up to
                                  steps_per_sync steps of every stepped Euler problem (each runs
                                  min(steps_per_sync, its remaining steps), so a round does not

@@ -47,6 +47,16 @@ constexpr int kBatchStagingDirect = 1;  // every thread loads from global memory
 constexpr int kBatchStagingWalk = 2;    // warps walk rows of units, no tile staging (batch_euler_walk_kernel)
 constexpr int kNumBatchStagings = 3;
 
+// The staging of per-step launches: FP32 problems walk in place of the TMA tile
+// pipeline, which is slower on every set tried (us a step, tiles / walks: one
+// 64^2 6.35 / 5.99, one 1000^2 30.9 / 13.4, 16 of 64-500 29.4 / 16.5, 64 of
+// 32-128 15.7 / 11.9, 512 of 32 16.2 / 16.0, 512 of 32-512 420 / 185).
+// Dependency-driven rounds keep the tiles (one 64^2 5.1 against 8.6).
+static int step_staging(ripple_dtype dt, int staging)
+{
+    return dt == RIPPLE_F32 && staging == kBatchStagingTma ? kBatchStagingWalk : staging;
+}
+
 template <typename T, int LAYOUT, int V>
 static cudaError_t step_v(int staging, int grid, cudaStream_t s, const BatchEuler* e, const void* f,
                           const int* table, BatchCtl* c, int kind, BatchAsync* q)
@@ -56,15 +66,17 @@ static cudaError_t step_v(int staging, int grid, cudaStream_t s, const BatchEule
     if (kind != 0)
         batch_fim_kernel<T><<<grid, EikTile<2>::NT, 0, s>>>(static_cast<const BatchFim<T>*>(f), table, c);
     else if (q && staging == kBatchStagingWalk)  // a dependency-driven round over walk units
-        batch_euler_walk_async_kernel<T><<<grid, kBatchWalkThreads, 0, s>>>(e, table, c, q);
+        batch_euler_walk_async_kernel<T, LAYOUT><<<grid, batch_walk_threads<T>(), batch_walk_smem<T>(), s>>>(e, table, c, q);
     else if (q)  // a dependency-driven round over tiles (TMA staging)
         batch_euler_kernel<T, LAYOUT, TX, TY, true><<<grid, BC::NTHREADS, BC::SMEM, s>>>(e, table, c, q);
     else if (staging == kBatchStagingDirect)
         batch_euler_direct_kernel<T, LAYOUT, TX, TY><<<grid, 256, 0, s>>>(e, table, c);
     else if (staging == kBatchStagingWalk)
-        batch_euler_walk_kernel<T><<<grid, kBatchWalkThreads, 0, s>>>(e, table, c);
-    else
+        batch_euler_walk_kernel<T, LAYOUT><<<grid, batch_walk_threads<T>(), batch_walk_smem<T>(), s>>>(e, table, c);
+    else if constexpr (std::is_same<T, double>::value)
         batch_euler_kernel<T, LAYOUT, TX, TY><<<grid, BC::NTHREADS, BC::SMEM, s>>>(e, table, c);
+    else
+        return cudaErrorInvalidValue;  // see step_staging
     return cudaGetLastError();
 }
 // CTAs per SM of the Euler step kernel of a staging (which also sets the TMA
@@ -81,16 +93,25 @@ static int occ_v(int staging)
     if (staging == kBatchStagingWalk) {
         // the per-step and the dependency-driven walk kernels share the grid
         int na = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_euler_walk_kernel<T>, kBatchWalkThreads, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&na, batch_euler_walk_async_kernel<T>, kBatchWalkThreads, 0);
+        auto k = batch_euler_walk_kernel<T, LAYOUT>;
+        auto ka = batch_euler_walk_async_kernel<T, LAYOUT>;
+        constexpr int sm = batch_walk_smem<T>(), nt = batch_walk_threads<T>();
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) != cudaSuccess) return 0;
+        if (cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) != cudaSuccess) return 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, nt, sm);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&na, ka, nt, sm);
         return std::min(n, na);
     }
     using BC = BatchEulerCfg<T, LAYOUT, TX, TY>;
-    auto k = batch_euler_kernel<T, LAYOUT, TX, TY, false>;
     auto ka = batch_euler_kernel<T, LAYOUT, TX, TY, true>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BC::SMEM) != cudaSuccess) return 0;
     if (cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, BC::SMEM) != cudaSuccess) return 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, BC::NTHREADS, BC::SMEM);
+    if constexpr (std::is_same<T, double>::value) {
+        auto k = batch_euler_kernel<T, LAYOUT, TX, TY, false>;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BC::SMEM) != cudaSuccess) return 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, BC::NTHREADS, BC::SMEM);
+    } else {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ka, BC::NTHREADS, BC::SMEM);
+    }
     return n;
 }
 template <typename T, int LAYOUT>
@@ -335,8 +356,9 @@ struct BatchRuntime {
     BatchAsync* h_async = nullptr;  // pinned staging of the control block
     int* h_cum = nullptr;           // pinned, [kMaxRoundSteps + 1]
     std::vector<Inst*> euler_order;  // Euler instances in table order (set by rebuild_tables)
+    int walk_rows = 16;  // rows of a walk unit (set by rebuild_tables)
     bool dirty = true;
-    bool small_only = false;  // batched rounds over the small Euler problems only (solo_round decides)
+    bool small_only = false;  // batched rounds over the (in FP64: small) Euler problems only (solo_round decides)
     bool has_e = false, has_f = false;  // resident kinds (set by rebuild_tables)
     long long gstep_e = 0;  // Euler steps issued (== device counter once they completed)
     long long gstep_f = 0;  // FIM iterations issued
@@ -733,18 +755,56 @@ static ripple_status grow(BatchRuntime* rt, int ne, int nf, int nt)
 
 // Rebuild the descriptor arrays and the tile table of the resident set.
 // Table entries of an instance: its tiles, or with walk staging its walk
-// units of kSoloW columns x kBatchWalkRows rows (per-step launches and
+// units of walk_cols() columns x rt->walk_rows rows (per-step launches and
 // dependency-driven rounds alike).
-static bool walk_units(const BatchRuntime* rt) { return rt->cfg.staging == kBatchStagingWalk; }
-static int walk_strips(const Inst* in) { return (int)((in->req.dims[0] + kSoloW - 1) / kSoloW); }
+static bool walk_units(const BatchRuntime* rt)
+{
+    const int sg = rt->cfg.async_queue ? rt->cfg.staging : step_staging(rt->cfg.dtype, rt->cfg.staging);
+    return sg == kBatchStagingWalk;
+}
+static int walk_cols(ripple_dtype dt) { return dt == RIPPLE_F32 ? batch_walk_cols<float>() : batch_walk_cols<double>(); }
+static int walk_strips(const BatchRuntime* rt, const Inst* in)
+{
+    const int c = walk_cols(rt->cfg.dtype);
+    return (int)((in->req.dims[0] + c - 1) / c);
+}
 static int table_entries(const BatchRuntime* rt, const Inst* in)
 {
     if (in->req.kind != RIPPLE_REQ_EULER || !walk_units(rt)) return in->ntiles;
-    return walk_strips(in) * (int)((in->req.dims[1] + kBatchWalkRows - 1) / kBatchWalkRows);
+    return walk_strips(rt, in) * (int)((in->req.dims[1] + rt->walk_rows - 1) / rt->walk_rows);
 }
+
+// Rows per walk unit for problems given as (strips, rows): the split of the
+// single-field walks (walk_split, runtime.cu) over several problems at once.
+// 512 problems of up to 512^2 take 24 (0.179 ms a step; 16 0.185, 8 0.215), 64
+// of at most 128^2 take 8 (11.7 us; 16 14.7), a single 64^2 one row.
+static int pick_walk_rows(const std::vector<std::pair<int, int>>& p, int sms)
+{
+    double best = 1e300;
+    int rows = 16;
+    for (int r : {1, 2, 3, 4, 6, 8, 12, 16, 24}) {
+        long long units = 0;
+        for (const auto& q : p) units += (long long)q.first * ((q.second + r - 1) / r);
+        const long long per = (units + 4 * sms - 1) / (4 * sms);
+        const double cost = units <= (long long)kWalkWarps * sms ? (r + 1.5) * std::max(1.0, 0.28 * (double)per)
+                                                                 : (r + 1.5) * ((double)units * 0.28 / (4.0 * sms) + 0.6);
+        if (cost < best) {
+            best = cost;
+            rows = r;
+        }
+    }
+    return rows;
+}
+
 
 static ripple_status rebuild_tables(BatchRuntime* rt)
 {
+    if (walk_units(rt)) {
+        std::vector<std::pair<int, int>> p;
+        for (const Inst* in : rt->resident)
+            if (in->req.kind == RIPPLE_REQ_EULER && in->active) p.emplace_back(walk_strips(rt, in), (int)in->req.dims[1]);
+        rt->walk_rows = pick_walk_rows(p, rt->ctx->sm_count);
+    }
     int ne = 0, nf = 0, nt = 0;
     for (Inst* in : rt->resident) {
         if (in->req.kind == RIPPLE_REQ_EULER && !in->active) continue;
@@ -783,7 +843,7 @@ static ripple_status rebuild_tables(BatchRuntime* rt)
             e.buf[1] = in->buf[1];
             e.ctl = &rt->slot_ctl[in->slot];
             e.g = in->g;
-            e.tiles_x = walk_units(rt) ? walk_strips(in) : in->tiles_x;
+            e.tiles_x = walk_units(rt) ? walk_strips(rt, in) : in->tiles_x;
             e.tile_begin = t;
             e.ntiles = table_entries(rt, in);
             e.bc = (int)in->req.fv.bc;
@@ -824,7 +884,7 @@ static ripple_status rebuild_tables(BatchRuntime* rt)
     if (nf)
         RIPPLE_CUDA(cudaMemcpyAsync(rt->d_fim, rt->h_fim, nf * fim_elem_size(rt->cfg.dtype), cudaMemcpyHostToDevice, s));
     if (nt) RIPPLE_CUDA(cudaMemcpyAsync(rt->d_table, rt->h_table, nt * sizeof(int), cudaMemcpyHostToDevice, s));
-    const int counts[2] = {nt_e, nt};
+    const int counts[3] = {nt_e, nt, rt->walk_rows};
     RIPPLE_CUDA(cudaMemcpyAsync(&rt->d_bctl->ntiles_e, counts, sizeof(counts), cudaMemcpyHostToDevice, s));
     RIPPLE_CUDA(cudaStreamSynchronize(s));  // counts live on this stack frame
     rt->has_e = ne > 0;
@@ -839,15 +899,16 @@ static ripple_status rebuild_tables(BatchRuntime* rt)
 static ripple_status launch_steps(BatchRuntime* rt, int K)
 {
     const int layout = rt->cfg.layout == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
+    const int staging = step_staging(rt->cfg.dtype, rt->cfg.staging);
     const int F = std::max(1, rt->cfg.fim_iters_per_step);
     auto unit = [&]() -> cudaError_t {
         cudaError_t e = cudaSuccess;
         if (rt->has_e)
-            e = launch_batch_step(rt->cfg.dtype, layout, rt->cfg.tile_variant, rt->cfg.staging, rt->grid,
+            e = launch_batch_step(rt->cfg.dtype, layout, rt->cfg.tile_variant, staging, rt->grid,
                                   rt->compute, rt->d_euler,
                                   rt->d_fim, rt->d_table, rt->d_bctl, 0);
         for (int f = 0; f < F && rt->has_f && e == cudaSuccess; ++f)
-            e = launch_batch_step(rt->cfg.dtype, layout, rt->cfg.tile_variant, rt->cfg.staging, rt->grid_fim,
+            e = launch_batch_step(rt->cfg.dtype, layout, rt->cfg.tile_variant, staging, rt->grid_fim,
                                   rt->compute, rt->d_euler,
                                   rt->d_fim, rt->d_table, rt->d_bctl, 1);
         return e;
@@ -946,7 +1007,8 @@ static ripple_status launch_round_async(BatchRuntime* rt, int K, std::vector<lon
     // so its next step is not held up behind one worker's chunk)
     const bool walk = walk_units(rt);
     const int grid = walk ? rt->grid : rt->grid_async;
-    const int workers = walk ? grid * (kBatchWalkThreads / 32) : grid;
+    const int nt = rt->cfg.dtype == RIPPLE_F32 ? batch_walk_threads<float>() : batch_walk_threads<double>();
+    const int workers = walk ? grid * (nt / 32) : grid;
     const int per_worker = (int)std::min<long long>(kAsyncChunk, (long long)rt->h_cum[1] / std::max(1, workers));
     a.chunk = std::max(1, per_worker);
     a.cum = rt->d_cum;
@@ -1015,14 +1077,21 @@ static void collect_finished(BatchRuntime* rt)
 // Requests arriving meanwhile are admitted after the round.  More resident
 // problems than that run in batched rounds, where one launch steps all of them.
 constexpr long long kSoloMaxSteps = 1024;
-// Euler problems of at least this many cells (512^2) run alone when they are
-// the oldest: alone a 1024^2 step takes 15 us, in a batched round with others
-// 33 us; smaller ones gain from sharing a batched launch
-constexpr long long kSoloBigCells = 1LL << 18;
+// FP64 Euler problems of at least this many cells (512^2) run alone when they
+// are the oldest; smaller ones, and FP32 ones of any size, gain from sharing a
+// batched launch (FP32 walks: a 1000^2 step takes 11 us alone and 13 us in a
+// batched launch, whose other problems come on top of it; 24 requests of up to
+// 1024^2, a third of them eikonal: 23.5 ms with the large ones alone, 18.0 ms)
+static long long solo_big_cells(ripple_dtype dt) { return dt == RIPPLE_F64 ? 1LL << 18 : INT64_MAX; }
+// FP32 problems of at least this many cells (400^2) run alone on the packed
+// walks, smaller ones on the scalar solver, whose one-row units make a shorter
+// chain per step (64^2 3.4 against 4.0, 256^2 4.1 / 4.6, 512^2 6.9 / 6.0, 1024^2
+// 15.4 / 11.2 us a step)
+constexpr long long kSoloWalkCells = 160000;
 
-// Solo GPU seconds an Euler step of `cells` cells takes (a fit of the
-// multi-step solver on GB300: a fixed barrier and dt cost, then the cells).
-static double solo_step_seconds(double cells) { return 3.3e-6 + 12e-12 * cells; }
+// Solo GPU seconds an FP32 Euler step of `cells` cells takes (a fit of the
+// multi-step solvers on GB300: a fixed barrier and dt cost, then the cells).
+static double solo_step_seconds(double cells) { return 3.5e-6 + 7.5e-12 * cells; }
 
 static ripple_status solo_round(BatchRuntime* rt, bool& handled)
 {
@@ -1036,10 +1105,10 @@ static ripple_status solo_round(BatchRuntime* rt, bool& handled)
         for (Inst* r : rt->resident)
             if (!in || r->t_submit < in->t_submit) in = r;
         // it runs alone while few problems are resident, and always when it is
-        // an eikonal problem or a large Euler one (large ones advance faster
-        // alone than in lockstep with others); otherwise the small Euler
-        // problems share batched rounds
-        const bool large = in->req.kind == RIPPLE_REQ_EIKONAL || in->req.dims[0] * in->req.dims[1] >= kSoloBigCells;
+        // an eikonal problem or a large FP64 Euler one; otherwise the Euler
+        // problems share batched rounds (in FP64 the small ones)
+        const bool large = in->req.kind == RIPPLE_REQ_EIKONAL ||
+                           in->req.dims[0] * in->req.dims[1] >= solo_big_cells(rt->cfg.dtype);
         small_only = rt->resident.size() > (size_t)rt->cfg.solo_rounds && !large;
     }
     if (small_only != rt->small_only) {
@@ -1082,46 +1151,59 @@ static ripple_status solo_round(BatchRuntime* rt, bool& handled)
         const double est_step = solo_step_seconds((double)cells);
         const long long K = std::min<long long>(
             r.nsteps - in->steps_done, std::max<long long>(8, std::min<long long>(kSoloMaxSteps, (long long)(1e-3 / est_step))));
-        SoloEuler a{};
-        a.buf[0] = in->buf[0];
-        a.buf[1] = in->buf[1];
-        a.ctl = ctl;
-        a.g = in->g;
-        a.bc = (int)r.fv.bc;
-        a.K = (int)K;
-        a.first = in->steps_done;
-        a.cfl = r.fv.cfl;
-        a.gamma = r.fv.gamma;
-        a.gm1 = r.fv.gamma - 1.0;
-        a.inv_dx0 = 1.0 / r.fv.dx[0];
-        a.inv_dx1 = 1.0 / r.fv.dx[1];
-        a.gamma_f = (float)a.gamma;
-        a.gm1_f = (float)a.gm1;
-        a.inv_dx0_f = (float)a.inv_dx0;
-        a.inv_dx1_f = (float)a.inv_dx1;
-        a.bar = rt->d_solo_bar;
-        a.spin_limit = grid_spin_limit();
-        a.err = &rt->d_bctl->err;
-        const int n0 = (int)r.dims[0], n1 = (int)r.dims[1];
-        const int per_sm = dt == RIPPLE_F32 ? rt->solo_occ[0] : rt->solo_occ[1];  // at kSoloThreads
-        const int sms = rt->ctx->sm_count;
-        a.strips = (n0 + kSoloW - 1) / kSoloW;
-        // segments as short as one row while the units fit one full CTA per SM
-        const long long most = (long long)sms * (kSoloThreads / 32);
-        a.rows = (int)std::min<long long>(n1, std::max<long long>(1, ((long long)n1 * a.strips + most - 1) / most));
-        a.segs = (n1 + a.rows - 1) / a.rows;
-        const long long units = (long long)a.strips * a.segs;
-        // CTAs of as few warps as spread the units over every SM (a small
-        // problem's step is then short chains on many SMs, not long ones on few)
-        const int wpc = (int)std::min<long long>(kSoloThreads / 32, std::max<long long>(1, (units + sms - 1) / sms));
-        const int grid = (int)std::max<long long>(
-            1, std::min<long long>((units + wpc - 1) / wpc, (long long)std::max(1, per_sm) * sms));
-        RIPPLE_CUDA(cudaMemsetAsync(rt->d_solo_bar, 0, 2 * sizeof(unsigned), s));
         RIPPLE_CUDA(cudaEventRecord(rt->ev_r0, s));
-        void* args[] = {&a};
-        const void* kern = dt == RIPPLE_F32 ? (const void*)solo_euler2d_kernel<float>
-                                            : (const void*)solo_euler2d_kernel<double>;
-        RIPPLE_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(32 * wpc), args, 0, s));
+        if (dt == RIPPLE_F32 && cells >= kSoloWalkCells) {
+            // the single-field walks on the instance's buffers and control block
+            WalkStep a{};
+            for (int b = 0; b < 2; ++b) a.buf[b] = static_cast<float*>(in->buf[b]);
+            a.ctl = ctl;
+            a.err = &rt->d_bctl->err;
+            a.K = (int)K;
+            a.cur = (int)(in->steps_done & 1);
+            a.slot = (int)(in->steps_done % 3);
+            a.first = in->steps_done == 0;
+            RIPPLE_CUDA(walk2d_solo_launch(rt->ctx, a, in->g, r.fv, rt->cfg.layout, s));
+        } else {
+            SoloEuler a{};
+            a.buf[0] = in->buf[0];
+            a.buf[1] = in->buf[1];
+            a.ctl = ctl;
+            a.g = in->g;
+            a.bc = (int)r.fv.bc;
+            a.K = (int)K;
+            a.first = in->steps_done;
+            a.cfl = r.fv.cfl;
+            a.gamma = r.fv.gamma;
+            a.gm1 = r.fv.gamma - 1.0;
+            a.inv_dx0 = 1.0 / r.fv.dx[0];
+            a.inv_dx1 = 1.0 / r.fv.dx[1];
+            a.gamma_f = (float)a.gamma;
+            a.gm1_f = (float)a.gm1;
+            a.inv_dx0_f = (float)a.inv_dx0;
+            a.inv_dx1_f = (float)a.inv_dx1;
+            a.bar = rt->d_solo_bar;
+            a.spin_limit = grid_spin_limit();
+            a.err = &rt->d_bctl->err;
+            const int n0 = (int)r.dims[0], n1 = (int)r.dims[1];
+            const int per_sm = dt == RIPPLE_F32 ? rt->solo_occ[0] : rt->solo_occ[1];  // at kSoloThreads
+            const int sms = rt->ctx->sm_count;
+            a.strips = (n0 + kSoloW - 1) / kSoloW;
+            // segments as short as one row while the units fit one full CTA per SM
+            const long long most = (long long)sms * (kSoloThreads / 32);
+            a.rows = (int)std::min<long long>(n1, std::max<long long>(1, ((long long)n1 * a.strips + most - 1) / most));
+            a.segs = (n1 + a.rows - 1) / a.rows;
+            const long long units = (long long)a.strips * a.segs;
+            // CTAs of as few warps as spread the units over every SM (a small
+            // problem's step is then short chains on many SMs, not long ones on few)
+            const int wpc = (int)std::min<long long>(kSoloThreads / 32, std::max<long long>(1, (units + sms - 1) / sms));
+            const int grid = (int)std::max<long long>(
+                1, std::min<long long>((units + wpc - 1) / wpc, (long long)std::max(1, per_sm) * sms));
+            RIPPLE_CUDA(cudaMemsetAsync(rt->d_solo_bar, 0, 2 * sizeof(unsigned), s));
+            void* args[] = {&a};
+            const void* kern = dt == RIPPLE_F32 ? (const void*)solo_euler2d_kernel<float>
+                                                : (const void*)solo_euler2d_kernel<double>;
+            RIPPLE_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(32 * wpc), args, 0, s));
+        }
         RIPPLE_CUDA(cudaEventRecord(rt->ev_r1, s));
         RIPPLE_CUDA(cudaMemcpyAsync(rt->h_berr, &rt->d_bctl->err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
         RIPPLE_CUDA(cudaEventRecord(rt->ev_step, s));
@@ -1173,7 +1255,7 @@ static ripple_status compute_round(BatchRuntime* rt)
         int64_t cells = 0;
         for (Inst* in : eu) {
             const int64_t c = in->req.dims[0] * in->req.dims[1];
-            const bool take = !(rt->small_only && c >= kSoloBigCells) &&
+            const bool take = !(rt->small_only && c >= solo_big_cells(rt->cfg.dtype)) &&
                               (budget <= 0 || cells == 0 || cells + c <= budget);
             if (take) cells += c;
             if (take != in->active) {
@@ -1447,7 +1529,8 @@ static ripple_status rt_start(BatchRuntime* rt)
     rt->free_slots.clear();
     for (int i = kSlots - 1; i >= 0; --i) rt->free_slots.push_back(i);
     const int layout = rt->cfg.layout == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
-    const int occ = std::max(1, batch_occupancy(rt->cfg.dtype, layout, rt->cfg.tile_variant, rt->cfg.staging));
+    const int occ = std::max(1, batch_occupancy(rt->cfg.dtype, layout, rt->cfg.tile_variant,
+                                                       step_staging(rt->cfg.dtype, rt->cfg.staging)));
     rt->grid = occ * rt->ctx->sm_count;
     rt->grid_fim = fim_occupancy(rt->cfg.dtype) * rt->ctx->sm_count;
     rt->grid_async =
@@ -1497,7 +1580,8 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
     for (int li = 0; li < 2 && status == RIPPLE_OK; ++li) {
         const ripple_layout lay = li == 0 ? RIPPLE_SOA : RIPPLE_AOS;
         for (int v = 0; v < kNumBatchVariants && status == RIPPLE_OK; ++v) {
-            const bool walk = sg == kBatchStagingWalk;  // walk units: the tile shape does not apply
+            const int run = step_staging(dt, sg);  // what a step of that staging runs
+            const bool walk = run == kBatchStagingWalk;  // walk units: the tile shape does not apply
             if (walk && v > 0) {
                 if (ms) ms[(sg * 2 + li) * kNumBatchVariants + v] = ms[(sg * 2 + li) * kNumBatchVariants];
                 continue;
@@ -1528,6 +1612,10 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
                 status = fail(RIPPLE_ERR_CUDA, "autotune: clearing control blocks");
                 break;
             }
+            std::vector<std::pair<int, int>> wp;
+            for (int i = 0; i < n; ++i)
+                wp.emplace_back((int)((sides[i] + walk_cols(dt) - 1) / walk_cols(dt)), (int)sides[i]);
+            const int walk_rows = pick_walk_rows(wp, ctx->sm_count);
             for (int i = 0; i < n && status == RIPPLE_OK; ++i) {
                 const int64_t dims[2] = {sides[i], sides[i]};
                 size_t bytes = 0;
@@ -1547,7 +1635,7 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
                 h[i].buf[1] = b[1];
                 h[i].ctl = ctl + i;
                 h[i].g = g;
-                h[i].tiles_x = walk ? (int)((sides[i] + kSoloW - 1) / kSoloW) : (int)((sides[i] + tx - 1) / tx);
+                h[i].tiles_x = walk ? (int)((sides[i] + walk_cols(dt) - 1) / walk_cols(dt)) : (int)((sides[i] + tx - 1) / tx);
                 h[i].tile_begin = (int)table.size();
                 h[i].bc = RIPPLE_BC_PERIODIC;
                 h[i].start_step = 0;
@@ -1560,7 +1648,7 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
                 h[i].gm1_f = (float)h[i].gm1;
                 h[i].inv_dx0_f = h[i].inv_dx1_f = (float)h[i].inv_dx0;
                 if (status == RIPPLE_OK) status = encode_batch_maps(h[i], lay, dt, v);
-                const int nt = walk ? h[i].tiles_x * (int)((sides[i] + kBatchWalkRows - 1) / kBatchWalkRows)
+                const int nt = walk ? h[i].tiles_x * (int)((sides[i] + walk_rows - 1) / walk_rows)
                                     : h[i].tiles_x * (int)((sides[i] + ty - 1) / ty);
                 for (int k = 0; k < nt; ++k) table.push_back(i << 1);
             }
@@ -1585,6 +1673,7 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
             BatchCtl hb{};
             hb.ntiles_e = (int)table.size();
             hb.ntiles = (int)table.size();
+            hb.walk_rows = walk_rows;
             cudaError_t ce = cudaMemcpyAsync(ctl, hc.data(), n * sizeof(FieldCtl), cudaMemcpyHostToDevice, s);
             if (ce == cudaSuccess)
                 ce = cudaMemcpyAsync(d_e, h.data(), n * sizeof(BatchEuler), cudaMemcpyHostToDevice, s);
@@ -1601,13 +1690,13 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
                 break;
             }
             const int lay_i = lay == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
-            const int grid = std::max(1, batch_occupancy(dt, lay_i, v, sg)) * ctx->sm_count;
+            const int grid = std::max(1, batch_occupancy(dt, lay_i, v, run)) * ctx->sm_count;
             for (int k = 0; k < 3 && ce == cudaSuccess; ++k)
-                ce = launch_batch_step(dt, lay_i, v, sg, grid, s, d_e, nullptr, d_t, d_c, 0);
+                ce = launch_batch_step(dt, lay_i, v, run, grid, s, d_e, nullptr, d_t, d_c, 0);
             cudaEventRecord(e0, s);
             const int reps = 6;
             for (int k = 0; k < reps && ce == cudaSuccess; ++k)
-                ce = launch_batch_step(dt, lay_i, v, sg, grid, s, d_e, nullptr, d_t, d_c, 0);
+                ce = launch_batch_step(dt, lay_i, v, run, grid, s, d_e, nullptr, d_t, d_c, 0);
             cudaEventRecord(e1, s);
             cudaStreamSynchronize(s);
             float el = 0.f;
@@ -1715,7 +1804,9 @@ ripple_status ripple_batch_configure(ripple_ctx ctx, const ripple_batch_config* 
             cfg->staging != rt->cfg.staging) {
             // the kernel grid depends on the variant; the scheduler re-reads it
             const int layout = cfg->layout == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
-            rt->grid = std::max(1, batch_occupancy(cfg->dtype, layout, cfg->tile_variant, cfg->staging)) * ctx->sm_count;
+            rt->grid = std::max(1, batch_occupancy(cfg->dtype, layout, cfg->tile_variant,
+                                                   step_staging(cfg->dtype, cfg->staging))) *
+                       ctx->sm_count;
             rt->grid_fim = fim_occupancy(cfg->dtype) * ctx->sm_count;
             rt->grid_async =
                 std::max(1, batch_occupancy(cfg->dtype, layout, cfg->tile_variant, kBatchStagingTma)) * ctx->sm_count;

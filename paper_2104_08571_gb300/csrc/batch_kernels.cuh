@@ -18,6 +18,7 @@
 #include "euler_sweep.cuh"
 #include "field.cuh"
 #include "fim_tile.cuh"
+#include "pair_math.cuh"
 
 namespace ripple {
 
@@ -46,6 +47,65 @@ __device__ __forceinline__ T field_const(double v, float vf)
     else return v;
 }
 
+// The arithmetic of the batched step.  An FP32 problem may be advanced by the
+// tiles below or by the walks (euler_walk2d.cuh, on packed cell pairs), in any
+// mixture, and its bits do not depend on which: the FP32 forms here round every
+// operation as the packed ones do (explicitly, so that nothing is contracted
+// differently) and, like them, carry twice the Rusanov flux, halved in the
+// update's dt.
+template <int D>
+__device__ __forceinline__ void batch_flux(const float (&q)[4], float gamma, float gm1, float (&F)[4], float& p, float& s)
+{
+    const float inv = rcp_v(q[0]);
+    const float mm = __fmaf_rn(q[2], q[2], __fmul_rn(q[1], q[1]));
+    p = __fmul_rn(gm1, __fmaf_rn(-0.5f, __fmul_rn(mm, inv), q[3]));
+    const float un = __fmul_rn(q[1 + D], inv);
+    F[0] = q[1 + D];
+    F[1] = D == 0 ? __fmaf_rn(q[1], un, p) : __fmul_rn(q[1], un);
+    F[2] = D == 1 ? __fmaf_rn(q[2], un, p) : __fmul_rn(q[2], un);
+    F[3] = __fmul_rn(__fadd_rn(q[3], p), un);
+    s = __fadd_rn(fabsf(un), sqrt_v(__fmul_rn(__fmul_rn(gamma, p), inv)));
+}
+template <typename T, int D>
+__device__ __forceinline__ void batch_face(const T (&a)[4], const T (&b)[4], T gamma, T gm1, T (&F)[4], T& chk,
+                                           bool valid)
+{
+    if constexpr (std::is_same<T, float>::value) {
+        float Fa[4], Fb[4], pa, pb, sa, sb;
+        batch_flux<D>(a, gamma, gm1, Fa, pa, sa);
+        batch_flux<D>(b, gamma, gm1, Fb, pb, sb);
+        track_min(chk, valid, a[0], pa, b[0], pb);
+        const float s = fmaxf(sa, sb);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) F[m] = __fmaf_rn(s, __fsub_rn(a[m], b[m]), __fadd_rn(Fa[m], Fb[m]));
+    } else {
+        rusanov<T, 2, D>(a, b, gamma, gm1, F, chk, valid);
+    }
+}
+template <typename T>
+__device__ __forceinline__ T batch_update(T q, T fxl, T fxr, T fyd, T fyu, T ix, T iy, T dt)
+{
+    if constexpr (std::is_same<T, float>::value)
+        return __fmaf_rn(-0.5f * dt, __fmaf_rn(__fsub_rn(fyu, fyd), iy, __fmul_rn(__fsub_rn(fxr, fxl), ix)), q);
+    else
+        return cell_update2(q, fxl, fxr, fyd, fyu, ix, iy, dt);
+}
+template <typename T>
+__device__ __forceinline__ T batch_wave_sum(const T (&q)[4], T gamma, T gm1, const T (&inv_dx)[3], bool& ok)
+{
+    if constexpr (std::is_same<T, float>::value) {
+        const float inv = rcp_v(q[0]);
+        const float mm = __fmaf_rn(q[2], q[2], __fmul_rn(q[1], q[1]));
+        const float p = __fmul_rn(gm1, __fmaf_rn(-0.5f, __fmul_rn(mm, inv), q[3]));
+        ok = (q[0] > 0.f) & (p > 0.f);
+        const float c = sqrt_v(__fmul_rn(__fmul_rn(gamma, p), inv));
+        const float s = __fmul_rn(__fadd_rn(fabsf(__fmul_rn(q[1], inv)), c), inv_dx[0]);
+        return __fmaf_rn(__fadd_rn(fabsf(__fmul_rn(q[2], inv)), c), inv_dx[1], s);
+    } else {
+        return wave_sum<T, 2>(q, gamma, gm1, inv_dx, ok);
+    }
+}
+
 // One resident 2D eikonal instance.
 template <typename T>
 struct BatchFim {
@@ -68,7 +128,9 @@ struct BatchCtl {
     unsigned int done[2];         // CTAs finished in the current launch of each kind
     int ntiles_e;                 // table entries [0, ntiles_e) are Euler tiles
     int ntiles;                   // entries [ntiles_e, ntiles) are eikonal tiles
+    int walk_rows;                // rows of a walk unit
     unsigned int err;             // DEV_ERR_TIMEOUT: a bounded wait of a batched launch ran out
+    unsigned int work;            // FP32 walk launches: units handed out beyond each warp's first; zero between launches
 };
 
 // Dependency-driven round of the batched Euler step (one persistent launch for
@@ -138,6 +200,7 @@ __device__ __forceinline__ void batch_finish_launch(BatchCtl* bctl, int kind, un
         __threadfence();
         if (atomicAdd(&bctl->done[kind], 1u) == gridDim.x - 1) {
             bctl->done[kind] = 0u;
+            if (kind == 0) bctl->work = 0u;
             __threadfence();
             atomicAdd(&bctl->gstep[kind], steps);
         }
@@ -391,7 +454,7 @@ __global__ void __launch_bounds__(288) batch_euler_kernel(const BatchEuler* __re
                     a[m] = S[o + m * SM];
                     b[m] = S[o + SX + m * SM];
                 }
-                rusanov<T, 2, 0>(a, b, gamma, gm1, F, chk, (x0 + fx <= g.n[0]) && (y0 + cy < g.n[1]));
+                batch_face<T, 0>(a, b, gamma, gm1, F, chk, (x0 + fx <= g.n[0]) && (y0 + cy < g.n[1]));
 #pragma unroll
                 for (int m = 0; m < NC; ++m) FX[m * NFX + it] = F[m];
             } else {
@@ -404,7 +467,7 @@ __global__ void __launch_bounds__(288) batch_euler_kernel(const BatchEuler* __re
                     a[m] = S[o + m * SM];
                     b[m] = S[o + SY + m * SM];
                 }
-                rusanov<T, 2, 1>(a, b, gamma, gm1, F, chk, (x0 + cx < g.n[0]) && (y0 + fy <= g.n[1]));
+                batch_face<T, 1>(a, b, gamma, gm1, F, chk, (x0 + cx < g.n[0]) && (y0 + fy <= g.n[1]));
 #pragma unroll
                 for (int m = 0; m < NC; ++m) FY[m * NFY + kk] = F[m];
             }
@@ -422,14 +485,14 @@ __global__ void __launch_bounds__(288) batch_euler_kernel(const BatchEuler* __re
             T qn[NC];
 #pragma unroll
             for (int m = 0; m < NC; ++m)
-                qn[m] = cell_update2(S[o + m * SM], FX[m * NFX + ly * (TX + 1) + lx], FX[m * NFX + ly * (TX + 1) + lx + 1],
+                qn[m] = batch_update(S[o + m * SM], FX[m * NFX + ly * (TX + 1) + lx], FX[m * NFX + ly * (TX + 1) + lx + 1],
                                      FY[m * NFY + ly * TX + lx], FY[m * NFY + (ly + 1) * TX + lx], inv_dx[0], inv_dx[1],
                                      dtT);
             const long long base = geom_cell(g, gx, gy, 0) * g.cell_stride;
 #pragma unroll
             for (int m = 0; m < NC; ++m) out[base + (long long)m * g.comp_stride] = qn[m];
             bool ok;
-            smax = wave_sum<T, 2>(qn, gamma, gm1, inv_dx, ok);
+            smax = batch_wave_sum<T>(qn, gamma, gm1, inv_dx, ok);
             bad |= !ok;
             if (gx < g.h || gx >= g.n[0] - g.h || gy < g.h || gy >= g.n[1] - g.h)
                 write_ghost_images<T, 2>(out, g, h.bc, gx, gy, 0, qn);
@@ -589,7 +652,7 @@ __global__ void __launch_bounds__(256) batch_euler_direct_kernel(const BatchEule
                     a[m] = S[m][cy + 1][fx];
                     b[m] = S[m][cy + 1][fx + 1];
                 }
-                rusanov<T, 2, 0>(a, b, gamma, gm1, F, chk, (x0 + fx <= g.n[0]) && (y0 + cy < g.n[1]));
+                batch_face<T, 0>(a, b, gamma, gm1, F, chk, (x0 + fx <= g.n[0]) && (y0 + cy < g.n[1]));
 #pragma unroll
                 for (int m = 0; m < NC; ++m) FX[m][it] = F[m];
             } else {
@@ -601,7 +664,7 @@ __global__ void __launch_bounds__(256) batch_euler_direct_kernel(const BatchEule
                     a[m] = S[m][fy][cx + 1];
                     b[m] = S[m][fy + 1][cx + 1];
                 }
-                rusanov<T, 2, 1>(a, b, gamma, gm1, F, chk, (x0 + cx < g.n[0]) && (y0 + fy <= g.n[1]));
+                batch_face<T, 1>(a, b, gamma, gm1, F, chk, (x0 + cx < g.n[0]) && (y0 + fy <= g.n[1]));
 #pragma unroll
                 for (int m = 0; m < NC; ++m) FY[m][kk] = F[m];
             }
@@ -614,13 +677,13 @@ __global__ void __launch_bounds__(256) batch_euler_direct_kernel(const BatchEule
             T qn[NC];
 #pragma unroll
             for (int m = 0; m < NC; ++m)
-                qn[m] = cell_update2(S[m][ly + 1][lx + 1], FX[m][ly * (TX + 1) + lx], FX[m][ly * (TX + 1) + lx + 1],
+                qn[m] = batch_update(S[m][ly + 1][lx + 1], FX[m][ly * (TX + 1) + lx], FX[m][ly * (TX + 1) + lx + 1],
                                      FY[m][ly * TX + lx], FY[m][(ly + 1) * TX + lx], inv_dx[0], inv_dx[1], dtT);
             const long long base = geom_cell(g, gx, gy, 0) * g.cell_stride;
 #pragma unroll
             for (int m = 0; m < NC; ++m) out[base + (long long)m * g.comp_stride] = qn[m];
             bool ok;
-            smax = wave_sum<T, 2>(qn, gamma, gm1, inv_dx, ok);
+            smax = batch_wave_sum<T>(qn, gamma, gm1, inv_dx, ok);
             bad |= !ok;
             if (gx < g.h || gx >= g.n[0] - g.h || gy < g.h || gy >= g.n[1] - g.h)
                 write_ghost_images<T, 2>(out, g, d.bc, gx, gy, 0, qn);

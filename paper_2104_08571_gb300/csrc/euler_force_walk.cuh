@@ -199,8 +199,8 @@ __device__ __forceinline__ void ForceWalk<DIM, LAYOUT, D, XS, LAST>::run(float* 
     }
     if constexpr (LAST) {
         const long long cstr = LAYOUT == LAYOUT_SOA ? cs : 1;
-        if (v0 && !nw.ok0) walk_bad_cell<DIM>(&a, po0, stride, cstr, D, x, line, r0, r1);
-        if (v1 && !nw.ok1) walk_bad_cell<DIM>(&a, po0 + CST, stride, cstr, D, x + 1, line, r0, r1);
+        if (v0 && !nw.ok0) walk_bad_cell<DIM>(a.ctl, a.gamma_f, a.gm1_f, po0, stride, cstr, D, x, line, r0, r1);
+        if (v1 && !nw.ok1) walk_bad_cell<DIM>(a.ctl, a.gamma_f, a.gm1_f, po0 + CST, stride, cstr, D, x + 1, line, r0, r1);
     }
 }
 
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_force_walk_kernel(co
         if (s + 1 < a.K && !grid_barrier(&ctl->bar[0], ++phase, a.spin_limit, sflag)) break;
     }
     if (sflag[0]) {
-        if (tid == 0) atomicOr(&ctl->err, DEV_ERR_TIMEOUT);
+        if (tid == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
         return;
     }
     walk_leave(ctl);

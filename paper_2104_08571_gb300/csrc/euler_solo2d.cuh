@@ -1,5 +1,7 @@
 // Multi-step solver of ONE 2D Euler problem (first-order Rusanov), the
-// single-problem kernel of the batch runtime's solo rounds.
+// single-problem kernel of the batch runtime's solo rounds in FP64 and for
+// small FP32 problems (larger ones run the multi-step walks of
+// euler_walk2d.cuh), and the walk kernels of the batched step.
 //
 // One cooperative launch advances the problem K steps; a bounded grid barrier
 // separates the steps.  Per launched step the field and batched step kernels
@@ -31,6 +33,7 @@
 #include <cstdint>
 
 #include "batch_kernels.cuh"
+#include "euler_walk2d.cuh"
 #include "grid_sync.cuh"
 
 namespace ripple {
@@ -93,7 +96,7 @@ __device__ __forceinline__ void solo_unit_begin(const FieldGeom& g, int strips, 
     solo_load(in, g, w.xl, w.y0, w.qc);
     solo_load(in, g, w.xl, w.y0 + 1, w.qa);  // y0 + 1 <= n[1]: at most the ghost row
     if (w.y0 + 2 <= g.n[1]) solo_load(in, g, w.xl, w.y0 + 2, w.qf);
-    rusanov<T, 2, 1>(qd, w.qc, gamma, gm1, w.Fb, w.chk, w.upd);
+    batch_face<T, 1>(qd, w.qc, gamma, gm1, w.Fb, w.chk, w.upd);
 }
 
 // Walk the started unit's rows: faces, update, stores, ghost images.
@@ -107,22 +110,22 @@ __device__ __forceinline__ void solo_unit_walk(const FieldGeom& g, int bc, const
         T qg[4];
         if (y + 3 <= g.n[1]) solo_load(in, g, w.xl, y + 3, qg);
         T Fa[4], Fl[4], Fr[4], left[4];
-        rusanov<T, 2, 1>(w.qc, w.qa, gamma, gm1, Fa, w.chk, w.upd);
+        batch_face<T, 1>(w.qc, w.qa, gamma, gm1, Fa, w.chk, w.upd);
 #pragma unroll
         for (int m = 0; m < 4; ++m) left[m] = __shfl_up_sync(0xffffffffu, w.qc[m], 1);
-        rusanov<T, 2, 0>(left, w.qc, gamma, gm1, Fl, w.chk, w.xface);
+        batch_face<T, 0>(left, w.qc, gamma, gm1, Fl, w.chk, w.xface);
 #pragma unroll
         for (int m = 0; m < 4; ++m) Fr[m] = __shfl_down_sync(0xffffffffu, Fl[m], 1);
         if (w.upd) {
             T qn[4];
 #pragma unroll
             for (int m = 0; m < 4; ++m)
-                qn[m] = cell_update2(w.qc[m], Fl[m], Fr[m], w.Fb[m], Fa[m], inv_dx[0], inv_dx[1], dtT);
+                qn[m] = batch_update(w.qc[m], Fl[m], Fr[m], w.Fb[m], Fa[m], inv_dx[0], inv_dx[1], dtT);
             const long long base = geom_cell(g, w.x, y, 0) * g.cell_stride;
 #pragma unroll
             for (int m = 0; m < 4; ++m) out[base + (long long)m * g.comp_stride] = qn[m];
             bool ok;
-            smax = max(smax, wave_sum<T, 2>(qn, gamma, gm1, inv_dx, ok));
+            smax = max(smax, batch_wave_sum<T>(qn, gamma, gm1, inv_dx, ok));
             w.bad |= !ok;
             if (w.x < g.h || w.x >= g.n[0] - g.h || y < g.h || y >= g.n[1] - g.h)
                 write_ghost_images<T, 2>(out, g, bc, w.x, y, 0, qn);
@@ -204,79 +207,108 @@ __global__ void __launch_bounds__(kSoloThreads) solo_euler2d_kernel(const SoloEu
 }
 
 // ---------------------------------------------------------------------------
-// The same row walks as the batched step (one launch per global step over
-// every active Euler problem): table entries [0, ntiles_e) of the batch are
-// walk units instead of tiles, instance-major (BatchEuler::tile_begin is the
-// instance's first unit, tiles_x its strips of kSoloW columns, units of
-// kBatchWalkRows rows).  A warp takes one unit at a time: the instance's local
-// step, its dt (lane 0, FP64, broadcast), the walk, its wave-speed maximum;
-// unit 0 of an instance advances t and clears the ring slot after next, as
-// tile 0 does in the tiled step.  Results are those of the tiled step bit for
-// bit (same faces, same update).
+// The row walks of the batched step (one launch per global step over every
+// active Euler problem): table entries [0, ntiles_e) of the batch are walk
+// units instead of tiles, instance-major (BatchEuler::tile_begin is the
+// instance's first unit, tiles_x its strips of batch_walk_cols() columns, units
+// of BatchCtl::walk_rows rows).  A warp takes one unit at a time: the instance's
+// local step, its dt (lane 0, FP64, broadcast), the walk, its wave-speed
+// maximum; unit 0 of an instance advances t and clears the ring slot after
+// next, as tile 0 does in the tiled step.  Results are those of the tiled step
+// bit for bit.  FP64 units are the solo solver's above; FP32 units are the
+// packed walks of the single-field step (euler_walk2d.cuh), 60 columns of cell
+// pairs staged through a ring in shared memory: bound by issue, and a pair
+// costs little more than the scalar walk's cell did (512 problems: 0.335 ->
+// 0.185 ms a step).  The host picks the rows of a unit for the resident set:
+// long ones for a large set, few for a small one, whose step is one unit long.
 // ---------------------------------------------------------------------------
-constexpr int kBatchWalkRows = 16;
-constexpr int kBatchWalkThreads = 256;  // threads per CTA of the batched walk kernels (8 warps)
-// CTAs per SM the FP32 walk kernels are compiled for: three (80 registers, a
-// few bytes of spills) ran the 512-problem step 15 % faster than two (98
-// registers); the FP64 kernels need about 150 registers and keep one
 template <typename T>
-constexpr int batch_walk_min_blocks() { return sizeof(T) == 4 ? 3 : 1; }
+__host__ __device__ constexpr bool batch_walk_packed() { return sizeof(T) == 4; }
+template <typename T>
+constexpr int batch_walk_cols() { return batch_walk_packed<T>() ? kWalkUse : kSoloW; }
+// FP32: 16 warps per CTA, one CTA per SM, as the single-field walks; FP64: 8 warps (about 150 registers)
+template <typename T>
+constexpr int batch_walk_threads() { return batch_walk_packed<T>() ? kWalkWarps * 32 : 256; }
+template <typename T>
+constexpr int batch_walk_smem() { return batch_walk_packed<T>() ? Walk2D<SCHEME_RUSANOV1>::SMEM : 0; }
 
 // One walk unit of a batched step: local unit lu of instance d at the
 // instance's local step `local` (dt by lane 0 in FP64, broadcast; unit 0
 // advances t and clears the ring slot after next, as tile 0 does in the tiled
 // step), then the unit's wave-speed maximum into the instance's next ring slot.
-template <typename T>
-__device__ __forceinline__ void batch_walk_unit(const BatchEuler& d, int lu, long long local, int lane)
+template <typename T, int LAYOUT>
+__device__ __forceinline__ void batch_walk_unit(const BatchEuler& d, int lu, int rows, long long local, int lane,
+                                                float* ring)
 {
     const int rs = (int)(local % 3);
     FieldCtl* ctl = d.ctl;
+    const T* in = static_cast<const T*>(d.buf[local & 1]);
+    T* out = static_cast<T*>(d.buf[(local & 1) ^ 1]);
+    PlaneWalk<SCHEME_RUSANOV1, LAYOUT> pw;
+    if constexpr (batch_walk_packed<T>()) {
+        // the unit's first rows are on their way while dt is formed
+        const int r0 = (lu / d.tiles_x) * rows;
+        pw.begin(in, d, (lu % d.tiles_x) * kWalkUse - 2, r0, min(d.g.n[1], r0 + rows), ring, lane);
+    }
     double dt = 0.0;
     if (lane == 0) dt = d.cfl / __longlong_as_double((long long)__ldcg(&ctl->smax[rs]));
-    dt = __shfl_sync(0xffffffffu, dt, 0);
     if (lu == 0 && lane == 0) {
         ctl->t = local == 0 ? dt : ctl->t + dt;
         ctl->dt_last = dt;
         ctl->smax[(rs + 2) % 3] = 0ull;
     }
-    const T dtT = (T)dt;
-    const T gamma = field_const<T>(d.gamma, d.gamma_f), gm1 = field_const<T>(d.gm1, d.gm1_f);
-    const T inv_dx[3] = {field_const<T>(d.inv_dx0, d.inv_dx0_f), field_const<T>(d.inv_dx1, d.inv_dx1_f), T(0)};
-    const T* in = static_cast<const T*>(d.buf[local & 1]);
-    T* out = static_cast<T*>(d.buf[(local & 1) ^ 1]);
-    SoloUnit<T> w;
-    solo_unit_begin(d.g, d.tiles_x, kBatchWalkRows, in, lu, lane, gamma, gm1, w);
-    T smax = T(0);
-    solo_unit_walk(d.g, d.bc, in, out, gamma, gm1, inv_dx, dtT, w, smax);
-    T v = smax;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const bool wbad = __any_sync(0xffffffffu, w.bad || !(w.chk > T(0)));
-    if (lane == 0) {
-        atomic_max_pos_double(&ctl->smax[(rs + 1) % 3], (double)v);
-        if (wbad) {
+    T v = T(0);
+    if constexpr (batch_walk_packed<T>()) {
+        const float dtf = __shfl_sync(0xffffffffu, (float)dt, 0);
+        Walk2DConsts k;
+        k.gamma = splat<f2>(d.gamma_f);
+        k.gm1 = splat<f2>(d.gm1_f);
+        k.ivx[0] = splat<f2>(d.inv_dx0_f);
+        k.ivx[1] = splat<f2>(d.inv_dx1_f);
+        k.ivx[2] = k.hdtdx[0] = k.hdtdx[1] = splat<f2>(0.f);
+        k.mdt = splat<f2>(-0.5f * dtf);
+        pw.run(out, d, ring, lane, k, v);  // reports non-admissible states itself
+    } else {
+        dt = __shfl_sync(0xffffffffu, dt, 0);
+        const T dtT = (T)dt;
+        const T gamma = field_const<T>(d.gamma, d.gamma_f), gm1 = field_const<T>(d.gm1, d.gm1_f);
+        const T inv_dx[3] = {field_const<T>(d.inv_dx0, d.inv_dx0_f), field_const<T>(d.inv_dx1, d.inv_dx1_f), T(0)};
+        SoloUnit<T> w;
+        solo_unit_begin(d.g, d.tiles_x, rows, in, lu, lane, gamma, gm1, w);
+        solo_unit_walk(d.g, d.bc, in, out, gamma, gm1, inv_dx, dtT, w, v);
+        if (__any_sync(0xffffffffu, w.bad || !(w.chk > T(0))) && lane == 0) {
             record_bad(ctl, BAD_STATE, w.strip * kSoloW, w.y0, 0);
             atomicOr(&ctl->err, DEV_ERR_NUMERIC);
         }
     }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) atomic_max_pos_double(&ctl->smax[(rs + 1) % 3], (double)v);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kBatchWalkThreads, batch_walk_min_blocks<T>())
+// Each warp's first unit is the one of its own number, the rest are handed out
+// by bctl->work (asked for before the unit in hand is walked).
+template <typename T, int LAYOUT>
+__global__ void __launch_bounds__(batch_walk_threads<T>(), 1)
     batch_euler_walk_kernel(const BatchEuler* __restrict__ euler, const int* __restrict__ table,
                             BatchCtl* __restrict__ bctl)
 {
+    extern __shared__ __align__(128) float wsm[];
     const unsigned long long gstep = __ldcg(&bctl->gstep[0]);
-    const int end = __ldcg(&bctl->ntiles_e);
-    const int lane = threadIdx.x & 31;
-    const int wpc = blockDim.x >> 5;
-    const int nwarps = gridDim.x * wpc;
-    for (int u = blockIdx.x * wpc + (threadIdx.x >> 5); u < end; u += nwarps) {
+    const int end = __ldcg(&bctl->ntiles_e), rows = __ldcg(&bctl->walk_rows);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarps = gridDim.x * (blockDim.x >> 5);
+    float* ring = wsm + warp * (Walk2D<SCHEME_RUSANOV1>::SLOTS * 64 * 4);
+    for (int u = warp * gridDim.x + blockIdx.x; u < end;) {
+        int next = 0;
+        if (lane == 0 && end > nwarps) next = nwarps + (int)atomicAdd(&bctl->work, 1u);
+        __syncwarp();
         const int inst = __ldg(&table[u]) >> 1;
         const BatchEuler& d = euler[inst];
         const long long local = (long long)gstep - d.start_step;
-        if (local < 0 || local >= d.nsteps) continue;
-        batch_walk_unit<T>(d, u - d.tile_begin, local, lane);
+        if (local >= 0 && local < d.nsteps) batch_walk_unit<T, LAYOUT>(d, u - d.tile_begin, rows, local, lane, ring);
+        u = end > nwarps ? __shfl_sync(0xffffffffu, next, 0) : end;
     }
     __syncwarp();
     batch_finish_launch(bctl, 0);
@@ -292,19 +324,22 @@ __global__ void __launch_bounds__(kBatchWalkThreads, batch_walk_min_blocks<T>())
 // every lane's stores (cells, ghost images, wave-speed maximum, unit 0's ring
 // slot) before lane 0's release add, which the waiting lane 0's acquire pairs
 // with; the waiting warp's barrier after that acquire orders its lanes' loads
-// (L2 loads, no stale L1 lines) after it.  A warp publishes every unit before
+// after it (the acquire also drops the SM's stale L1 lines).  A warp publishes every unit before
 // it takes or waits for the next, and the tasks a wait needs precede it in the
 // order and were taken by running warps, so the waits end; a wait that runs
 // out stops its warp and reports DEV_ERR_TIMEOUT.  Each unit's arithmetic is
 // the per-step walk kernel's, so results are those of per-step launches bit
 // for bit.
-template <typename T>
-__global__ void __launch_bounds__(kBatchWalkThreads, batch_walk_min_blocks<T>())
+template <typename T, int LAYOUT>
+__global__ void __launch_bounds__(batch_walk_threads<T>(), 1)
     batch_euler_walk_async_kernel(const BatchEuler* __restrict__ euler, const int* __restrict__ table,
                                   BatchCtl* __restrict__ bctl, BatchAsync* __restrict__ q)
 {
     const unsigned long long gstep = __ldcg(&bctl->gstep[0]);
+    const int rows = __ldcg(&bctl->walk_rows);
+    extern __shared__ __align__(128) float wsm[];
     const int lane = threadIdx.x & 31;
+    float* ring = wsm + (threadIdx.x >> 5) * (Walk2D<SCHEME_RUSANOV1>::SLOTS * 64 * 4);
     const int total = q->total, chunk = q->chunk, K = q->K;
     bool ok = true;
     // the current chunk of tasks [c_lo, c_hi), the cached task range [s_lo, s_hi) of round step s_n
@@ -348,7 +383,7 @@ __global__ void __launch_bounds__(kBatchWalkThreads, batch_walk_min_blocks<T>())
                 break;
             }
         }
-        batch_walk_unit<T>(d, t - d.tile_begin, (long long)gstep + s_n - d.start_step, lane);
+        batch_walk_unit<T, LAYOUT>(d, t - d.tile_begin, rows, (long long)gstep + s_n - d.start_step, lane, ring);
         __syncwarp();
         if (lane == 0) red_release_gpu_add(&q->done[inst], 1u);
     }

@@ -47,7 +47,9 @@ __device__ __forceinline__ void rus2_pre(const f2 (&a)[4], const f2 (&b)[4], con
 }
 
 // One walk: rows r0 .. r1 - 1 of the strip whose lanes start at column x0.
-// begin() stages the walk's first rows, which needs no dt; run() walks.
+// begin() stages the walk's first rows, which needs no dt; run() walks.  `a`
+// describes the problem (g, bc, ctl, gamma_f, gm1_f): a WalkStep, or an
+// instance of the batched step.
 template <int SCHEME, int LAYOUT>
 struct PlaneWalk {
     static constexpr bool MH = SCHEME == SCHEME_MUSCL;
@@ -57,7 +59,8 @@ struct PlaneWalk {
     WalkRows rows;
     int x0, r0, r1;
 
-    __device__ __forceinline__ void begin(const float* __restrict__ in, const WalkStep& a, int x0_, int r0_, int r1_,
+    template <class A>
+    __device__ __forceinline__ void begin(const float* __restrict__ in, const A& a, int x0_, int r0_, int r1_,
                                           float* ring, int lane)
     {
         const FieldGeom& g = a.g;
@@ -77,12 +80,14 @@ struct PlaneWalk {
         }
     }
 
-    __device__ __forceinline__ void run(float* __restrict__ out, const WalkStep& a, float* ring, int lane,
+    template <class A>
+    __device__ __forceinline__ void run(float* __restrict__ out, const A& a, float* ring, int lane,
                                         const Walk2DConsts& k, float& smax);
 };
 
 template <int SCHEME, int LAYOUT>
-__device__ __forceinline__ void PlaneWalk<SCHEME, LAYOUT>::run(float* __restrict__ out, const WalkStep& a, float* ring,
+template <class A>
+__device__ __forceinline__ void PlaneWalk<SCHEME, LAYOUT>::run(float* __restrict__ out, const A& a, float* ring,
                                                                int lane, const Walk2DConsts& k, float& smax)
 {
     const FieldGeom& g = a.g;
@@ -206,8 +211,8 @@ __device__ __forceinline__ void PlaneWalk<SCHEME, LAYOUT>::run(float* __restrict
         atomicOr(&a.ctl->err, DEV_ERR_NUMERIC);
     }
     const long long cstr = LAYOUT == LAYOUT_SOA ? cs : 1;
-    if (v0 && !nw.ok0) walk_bad_cell<2>(&a, po0, stride, cstr, 1, x, 0, r0, r1);
-    if (v1 && !nw.ok1) walk_bad_cell<2>(&a, po0 + CST, stride, cstr, 1, x + 1, 0, r0, r1);
+    if (v0 && !nw.ok0) walk_bad_cell<2>(a.ctl, a.gamma_f, a.gm1_f, po0, stride, cstr, 1, x, 0, r0, r1);
+    if (v1 && !nw.ok1) walk_bad_cell<2>(a.ctl, a.gamma_f, a.gm1_f, po0 + CST, stride, cstr, 1, x + 1, 0, r0, r1);
 }
 
 template <int SCHEME, int LAYOUT>
@@ -264,7 +269,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_walk2d_kernel(const 
         if (s + 1 < a.K && !grid_barrier(&ctl->bar[0], (unsigned)(s + 1), a.spin_limit, sflag)) break;
     }
     if (sflag[0]) {
-        if (tid == 0) atomicOr(&ctl->err, DEV_ERR_TIMEOUT);
+        if (tid == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
         return;
     }
     walk_leave(ctl);

@@ -304,6 +304,82 @@ int sweep_occ(ripple_dtype dt, int dim, int layout, int scheme, int v)
     return dim == 2 ? sweep_occ_f64_2d(layout, scheme, v) : sweep_occ_f64_3d(layout, scheme, v);
 }
 
+// Rows per walk for `lines` independent lines of n rows on `sms` SMs of 16
+// resident warps, a walk of R rows costing R + extra.  In units of the time a
+// warp alone takes for a row, a scheduler with enough warps finishes a row
+// every 0.28 (a warp issues about every fourth cycle).  Walks that all have a
+// warp of their own end together; otherwise the last one handed out ends about
+// 0.6 walks after the schedulers have run out of others.  `most` bounds R:
+// walks along z keep as many planes in flight as they are long and lose L2
+// hits (200 x 171 x 186: 8 planes 149 us a step, 31 190, 62 223), and long
+// in-plane walks of a 3D field do the same (24 rows).
+static void walk_split(long long lines, int n, int sms, double extra, int most, int* rows, int* segs)
+{
+    double best = 1e300;
+    *rows = n;
+    *segs = 1;
+    for (int r = 1; r <= std::min(n, most); ++r) {
+        const int sg = (n + r - 1) / r;
+        const long long units = lines * sg, per = (units + 4 * sms - 1) / (4 * sms);  // walks per scheduler
+        const double cost = units <= (long long)kWalkWarps * sms
+                                ? (r + extra) * std::max(1.0, 0.28 * (double)per)
+                                : (r + extra) * ((double)units * 0.28 / (4.0 * sms) + 0.6);
+        if (cost < best) {
+            best = cost;
+            *rows = r;
+            *segs = sg;
+        }
+    }
+}
+
+// Steps of a walk launch: about 64 M cell updates, so that a launch stays near
+// a millisecond (a long call is then cut into several launches).
+static int walk_steps(const FieldGeom& g, int64_t left)
+{
+    const long long cells = (long long)g.n[0] * g.n[1] * g.n[2];
+    return (int)std::min<long long>(left, std::max(1LL, std::min(256LL, (64LL << 20) / cells)));
+}
+
+// Geometry, parameters and work split of a walk launch; returns its grid.
+static int walk_plan(const ripple_ctx_s* ctx, WalkStep& a, const FieldGeom& g, int scheme, double gamma, double cfl,
+                     const double* dx, int bc, int occ)
+{
+    const bool d3 = g.ndim == 3;
+    const int sms = ctx->sm_count;
+    a.g = g;
+    a.cfl = cfl;
+    a.gamma_f = (float)gamma;
+    a.gm1_f = (float)(gamma - 1.0);
+    for (int d = 0; d < g.ndim; ++d) {
+        a.inv_dx[d] = 1.0 / dx[d];
+        a.dx_cfl[d] = dx[d] / cfl;
+        a.inv_dx_f[d] = (float)a.inv_dx[d];
+    }
+    a.bc = bc;
+    a.spin_limit = grid_spin_limit();
+    a.strips = (g.n[0] + kWalkUse - 1) / kWalkUse;
+    walk_split((long long)a.strips * g.n[2], g.n[1], sms, scheme == SCHEME_RUSANOV1 ? 1.5 : 2.0, d3 ? 24 : 128, &a.rows,
+               &a.segs);
+    // unit numbers are 32-bit: at most 2^32 padded cells and at least 60 cells per unit row
+    long long units = (long long)a.strips * a.segs * g.n[2];
+    if (d3) {
+        a.zstrips = (g.n[0] + 63) / 64;
+        walk_split((long long)a.zstrips * g.n[1], g.n[2], sms, 1.0, 8, &a.zrows, &a.zsegs);
+        units = std::max(units, (long long)a.zstrips * g.n[1] * a.zsegs);
+    }
+    return (int)std::min<long long>((long long)occ * sms, units);
+}
+
+cudaError_t walk2d_solo_launch(ripple_ctx ctx, WalkStep& a, const FieldGeom& g, const ripple_fv_params& p,
+                               ripple_layout layout, cudaStream_t s)
+{
+    const int lay = layout == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
+    const int occ = walk2d_occ_f32(SCHEME_RUSANOV1, lay);
+    if (occ <= 0) return cudaErrorInvalidValue;
+    const int grid = walk_plan(ctx, a, g, SCHEME_RUSANOV1, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
+    return walk2d_launch_f32(SCHEME_RUSANOV1, lay, a, grid, s);
+}
+
 }  // namespace ripple
 
 using namespace ripple;
@@ -562,45 +638,9 @@ ripple_status ripple_field_set_sweep(ripple_field f, int variant, int zchunk)
     return RIPPLE_OK;
 }
 
-// Rows per walk for `lines` independent lines of n rows on `sms` SMs of 16
-// resident warps, a walk of R rows costing R + extra.  In units of the time a
-// warp alone takes for a row, a scheduler with enough warps finishes a row
-// every 0.28 (a warp issues about every fourth cycle).  Walks that all have a
-// warp of their own end together; otherwise the last one handed out ends about
-// 0.6 walks after the schedulers have run out of others.  `most` bounds R:
-// walks along z keep as many planes in flight as they are long and lose L2
-// hits (200 x 171 x 186: 8 planes 149 us a step, 31 190, 62 223), and long
-// in-plane walks of a 3D field do the same (24 rows).
-static void walk_split(long long lines, int n, int sms, double extra, int most, int* rows, int* segs)
-{
-    double best = 1e300;
-    *rows = n;
-    *segs = 1;
-    for (int r = 1; r <= std::min(n, most); ++r) {
-        const int sg = (n + r - 1) / r;
-        const long long units = lines * sg, per = (units + 4 * sms - 1) / (4 * sms);  // walks per scheduler
-        const double cost = units <= (long long)kWalkWarps * sms
-                                ? (r + extra) * std::max(1.0, 0.28 * (double)per)
-                                : (r + extra) * ((double)units * 0.28 / (4.0 * sms) + 0.6);
-        if (cost < best) {
-            best = cost;
-            *rows = r;
-            *segs = sg;
-        }
-    }
-}
-
-// Steps of a walk launch: about 64 M cell updates, so that a launch stays near
-// a millisecond (a long call is then cut into several launches).
-static int walk_steps(const FieldGeom& g, int64_t left)
-{
-    const long long cells = (long long)g.n[0] * g.n[1] * g.n[2];
-    return (int)std::min<long long>(left, std::max(1LL, std::min(256LL, (64LL << 20) / cells)));
-}
-
 // Steps of an FP32 field on strip walks: every 2D scheme, and the split FORCE
 // step in 3D.
-static ripple_status walk_field_steps(ripple_field U, const SweepParams& prm, int scheme, int layout, int64_t nsteps)
+static ripple_status walk_field_steps(ripple_field U, const ripple_fv_params& p, int scheme, int layout, int64_t nsteps)
 {
     ripple_ctx ctx = U->ctx;
     const FieldGeom& g = U->geom;
@@ -610,33 +650,11 @@ static ripple_status walk_field_steps(ripple_field U, const SweepParams& prm, in
                     : force ? force_walk_occ_f32_2d(layout)
                             : walk2d_occ_f32(scheme, layout);
     if (occ <= 0) return fail(RIPPLE_ERR_INTERNAL, "walk kernel does not fit");
-    const int ctas = occ * ctx->sm_count;
     WalkStep a{};
-    a.buf[0] = static_cast<float*>(U->buf[0]);
-    a.buf[1] = static_cast<float*>(U->buf[1]);
+    for (int b = 0; b < 2; ++b) a.buf[b] = static_cast<float*>(U->buf[b]);
     a.ctl = U->ctl;
-    a.g = g;
-    a.cfl = prm.cfl;
-    a.gamma_f = prm.gamma_f;
-    a.gm1_f = prm.gm1_f;
-    for (int d = 0; d < 3; ++d) {
-        a.inv_dx[d] = prm.inv_dx[d];
-        a.dx_cfl[d] = prm.inv_dx[d] > 0.0 ? 1.0 / (prm.inv_dx[d] * prm.cfl) : 0.0;
-        a.inv_dx_f[d] = prm.inv_dx_f[d];
-    }
-    a.bc = prm.bc;
-    a.spin_limit = grid_spin_limit();
-    a.strips = (g.n[0] + kWalkUse - 1) / kWalkUse;
-    walk_split((long long)a.strips * g.n[2], g.n[1], ctx->sm_count,
-               scheme == SCHEME_RUSANOV1 ? 1.5 : 2.0, d3 ? 24 : 128, &a.rows, &a.segs);
-    long long units = (long long)a.strips * a.segs * g.n[2];
-    if (d3) {
-        a.zstrips = (g.n[0] + 63) / 64;
-        walk_split((long long)a.zstrips * g.n[1], g.n[2], ctx->sm_count, 1.0, 8, &a.zrows, &a.zsegs);
-        units = std::max(units, (long long)a.zstrips * g.n[1] * a.zsegs);
-    }
-    // unit numbers are 32-bit: at most 2^32 padded cells and at least 60 cells per unit row
-    const int grid = (int)std::min<long long>(ctas, units);
+    a.err = &U->ctl->err;
+    const int grid = walk_plan(ctx, a, g, scheme, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
     for (int64_t done = 0; done < nsteps;) {
         a.K = walk_steps(g, nsteps - done);
         a.cur = U->cur;
@@ -784,7 +802,7 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     // FP32 fields: the 2D schemes and the split step run on strip walks (no
     // tile staging, several steps per launch) unless a kernel was chosen
     if (U->dtype == RIPPLE_F32 && U->variant < 0 && (U->ndim == 2 || split)) {
-        st = walk_field_steps(U, L.prm, scheme, layout, nsteps);
+        st = walk_field_steps(U, *p, scheme, layout, nsteps);
         if (st != RIPPLE_OK) return st;
         nsteps_left = 0;
     }

@@ -97,6 +97,10 @@ int force_walk_occ_f32_3d(int layout);
 // The same for the FP32 2D unsplit schemes (euler_walk2d.cuh), one launch for several steps.
 cudaError_t walk2d_launch_f32(int scheme, int layout, const WalkStep& a, int grid, cudaStream_t s);
 int walk2d_occ_f32(int scheme, int layout);
+// K first-order steps of one FP32 2D problem of geometry g (a.buf, ctl, err, K,
+// cur, slot and first set; the rest is filled in), queued on s (runtime.cu).
+cudaError_t walk2d_solo_launch(ripple_ctx ctx, WalkStep& a, const FieldGeom& g, const ripple_fv_params& p,
+                               ripple_layout layout, cudaStream_t s);
 
 // Aux kernels (f32/f64 x 2D/3D), defined in aux.cu; cap: most blocks of a launch.
 cudaError_t launch_prep(int dtype, int dim, void* buf, FieldCtl* ctl, const FieldGeom& g, int bc, double gamma,

@@ -37,6 +37,7 @@ struct WalkStep {
     int strips, rows, segs;     // in-plane walks: strips of columns, segments of `rows` rows
     int zstrips, zrows, zsegs;  // walks along z (3D split step)
     unsigned spin_limit;   // polls of a barrier wait before it gives up
+    unsigned* err;         // DEV_ERR_TIMEOUT when a barrier wait ran out
 };
 
 // The launch's grid barriers count up ctl->bar[0] (grid_sync.cuh); the last CTA
@@ -143,21 +144,22 @@ struct WalkNew {
 // Report the first non-admissible new state of a column (rare, out of line):
 // rows r0 .. r1 - 1 along `axis` of the column at element pointer p (row r0).
 template <int DIM>
-static __device__ __noinline__ void walk_bad_cell(const WalkStep* a, const float* p, long long stride, long long cstr,
-                                                  int axis, int x, int line, int r0, int r1)
+static __device__ __noinline__ void walk_bad_cell(FieldCtl* ctl, float gamma, float gm1, const float* p,
+                                                  long long stride, long long cstr, int axis, int x, int line, int r0,
+                                                  int r1)
 {
     for (int r = r0; r < r1; ++r, p += stride) {
         float q[DIM + 2];
         for (int m = 0; m < DIM + 2; ++m) q[m] = p[m * cstr];
         const float ivx[3] = {1.f, 1.f, 1.f};
         bool ok;
-        wave_sum<float, DIM>(q, a->gamma_f, a->gm1_f, ivx, ok);
+        wave_sum<float, DIM>(q, gamma, gm1, ivx, ok);
         if (!ok) {
-            record_bad(a->ctl, BAD_CELL, x, axis == 1 ? r : line, axis == 1 ? line : r);
+            record_bad(ctl, BAD_CELL, x, axis == 1 ? r : line, axis == 1 ? line : r);
             break;
         }
     }
-    atomicOr(&a->ctl->err, DEV_ERR_NUMERIC);
+    atomicOr(&ctl->err, DEV_ERR_NUMERIC);
 }
 
 // Store the updated pair of cells (x, x + 1) at element pointer p; v0, v1: the
