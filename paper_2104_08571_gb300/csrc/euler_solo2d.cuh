@@ -26,7 +26,7 @@
 // The step is the batched step's, term for term: dt = cfl / smax of the input
 // state (FP64, from the instance's 3-slot ring), the same Rusanov faces of the
 // same left/right states (a face's value depends only on its two states), the
-// same cell update (cell_update2), ghost images and wave-speed maximum.  A
+// same cell update (batch_update), ghost images and wave-speed maximum.  A
 // problem's state is therefore bitwise the same whichever kernel advanced
 // which of its steps.
 #pragma once

@@ -341,13 +341,14 @@ static int walk_steps(const FieldGeom& g, int64_t left)
 }
 
 // Geometry, parameters and work split of a walk launch; returns its grid.
-static int walk_plan(const ripple_ctx_s* ctx, WalkStep& a, const FieldGeom& g, int scheme, double gamma, double cfl,
-                     const double* dx, int bc, int occ)
+static int walk_plan(const ripple_ctx_s* ctx, WalkStep& a, const FieldGeom& g, bool f64, int scheme, double gamma,
+                     double cfl, const double* dx, int bc, int occ)
 {
     const bool d3 = g.ndim == 3;
     const int sms = ctx->sm_count;
     a.g = g;
     a.cfl = cfl;
+    a.gamma = gamma;
     a.gamma_f = (float)gamma;
     a.gm1_f = (float)(gamma - 1.0);
     for (int d = 0; d < g.ndim; ++d) {
@@ -357,6 +358,10 @@ static int walk_plan(const ripple_ctx_s* ctx, WalkStep& a, const FieldGeom& g, i
     }
     a.bc = bc;
     a.spin_limit = grid_spin_limit();
+    if (f64) {
+        tile64_plan(a, sms);
+        return (int)std::min<long long>((long long)occ * sms, (long long)a.strips * a.segs);
+    }
     a.strips = (g.n[0] + kWalkUse - 1) / kWalkUse;
     walk_split((long long)a.strips * g.n[2], g.n[1], sms, scheme == SCHEME_RUSANOV1 ? 1.5 : 2.0, d3 ? 24 : 128, &a.rows,
                &a.segs);
@@ -376,7 +381,7 @@ cudaError_t walk2d_solo_launch(ripple_ctx ctx, WalkStep& a, const FieldGeom& g, 
     const int lay = layout == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
     const int occ = walk2d_occ_f32(SCHEME_RUSANOV1, lay);
     if (occ <= 0) return cudaErrorInvalidValue;
-    const int grid = walk_plan(ctx, a, g, SCHEME_RUSANOV1, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
+    const int grid = walk_plan(ctx, a, g, false, SCHEME_RUSANOV1, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
     return walk2d_launch_f32(SCHEME_RUSANOV1, lay, a, grid, s);
 }
 
@@ -638,15 +643,17 @@ ripple_status ripple_field_set_sweep(ripple_field f, int variant, int zchunk)
     return RIPPLE_OK;
 }
 
-// Steps of an FP32 field on strip walks: every 2D scheme, and the split FORCE
-// step in 3D.
+// Steps of a field by the multi-step kernels: FP32 strip walks (every 2D
+// scheme, and the split FORCE step in 3D) and the FP64 first-order 2D tiles.
 static ripple_status walk_field_steps(ripple_field U, const ripple_fv_params& p, int scheme, int layout, int64_t nsteps)
 {
     ripple_ctx ctx = U->ctx;
     const FieldGeom& g = U->geom;
     const bool force = scheme == SCHEME_FORCE;
     const bool d3 = U->ndim == 3;  // FORCE only
-    const int occ = d3      ? force_walk_occ_f32_3d(layout)
+    const bool f64 = U->dtype == RIPPLE_F64;  // first-order 2D only
+    const int occ = f64     ? tile64_occ()
+                    : d3      ? force_walk_occ_f32_3d(layout)
                     : force ? force_walk_occ_f32_2d(layout)
                             : walk2d_occ_f32(scheme, layout);
     if (occ <= 0) return fail(RIPPLE_ERR_INTERNAL, "walk kernel does not fit");
@@ -654,13 +661,14 @@ static ripple_status walk_field_steps(ripple_field U, const ripple_fv_params& p,
     for (int b = 0; b < 2; ++b) a.buf[b] = static_cast<float*>(U->buf[b]);
     a.ctl = U->ctl;
     a.err = &U->ctl->err;
-    const int grid = walk_plan(ctx, a, g, scheme, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
+    const int grid = walk_plan(ctx, a, g, f64, scheme, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
     for (int64_t done = 0; done < nsteps;) {
         a.K = walk_steps(g, nsteps - done);
         a.cur = U->cur;
         a.slot = (int)(U->steps_total % 3);
         a.first = done == 0;
-        RIPPLE_CUDA(d3      ? force_walk_launch_f32_3d(layout, a, grid, ctx->stream)
+        RIPPLE_CUDA(f64     ? tile64_launch(a, grid, ctx->stream)
+                    : d3    ? force_walk_launch_f32_3d(layout, a, grid, ctx->stream)
                     : force ? force_walk_launch_f32_2d(layout, a, grid, ctx->stream)
                             : walk2d_launch_f32(scheme, layout, a, grid, ctx->stream));
         if (!d3) U->cur = (U->cur + a.K) & 1;  // 3D: the z walks bring the state back
@@ -799,9 +807,12 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     // each sweep writes the ghost images its successor reads; all read the same dt)
     const int sweeps = split ? U->ndim : 1;
     int64_t nsteps_left = nsteps;
-    // FP32 fields: the 2D schemes and the split step run on strip walks (no
-    // tile staging, several steps per launch) unless a kernel was chosen
-    if (U->dtype == RIPPLE_F32 && U->variant < 0 && (U->ndim == 2 || split)) {
+    // several steps per launch unless a kernel was chosen: FP32 2D schemes and
+    // the split step on strip walks; FP64 first-order 2D on compute-spread tiles
+    // (per step, tiles of euler_sweep.cuh -> now: 64^2 17.5 -> 7.4 us, 256^2
+    // 36 -> 19.7 us, 1024^2 380 -> 240 us)
+    const bool walks = U->dtype == RIPPLE_F32 ? U->ndim == 2 || split : U->ndim == 2 && scheme == SCHEME_RUSANOV1;
+    if (walks && U->variant < 0) {
         st = walk_field_steps(U, *p, scheme, layout, nsteps);
         if (st != RIPPLE_OK) return st;
         nsteps_left = 0;

@@ -97,6 +97,11 @@ int force_walk_occ_f32_3d(int layout);
 // The same for the FP32 2D unsplit schemes (euler_walk2d.cuh), one launch for several steps.
 cudaError_t walk2d_launch_f32(int scheme, int layout, const WalkStep& a, int grid, cudaStream_t s);
 int walk2d_occ_f32(int scheme, int layout);
+// The same for the first-order scheme on FP64 2D fields, either layout
+// (euler_tile64.cuh); tile64_plan sets the tile's sides and the tile counts.
+cudaError_t tile64_launch(const WalkStep& a, int grid, cudaStream_t s);
+int tile64_occ();
+void tile64_plan(WalkStep& a, int sms);
 // K first-order steps of one FP32 2D problem of geometry g (a.buf, ctl, err, K,
 // cur, slot and first set; the rest is filled in), queued on s (runtime.cu).
 cudaError_t walk2d_solo_launch(ripple_ctx ctx, WalkStep& a, const FieldGeom& g, const ripple_fv_params& p,

@@ -22,10 +22,10 @@ constexpr int kWalkUse = 60;   // columns updated by a walk that works along x t
 
 // Arguments of a multi-step walk launch.
 struct WalkStep {
-    float* buf[2];
+    float* buf[2];         // (FP64 tiles: doubles)
     FieldCtl* ctl;
     FieldGeom g;
-    double cfl;
+    double cfl, gamma;
     double inv_dx[3];
     double dx_cfl[3];      // dx / cfl: dx / dt is that times the largest wave-speed sum
     float gamma_f, gm1_f, inv_dx_f[3];
@@ -35,6 +35,7 @@ struct WalkStep {
     int slot;              // wave-speed ring slot of that state
     int first;             // the first step of a call: t = dt instead of t += dt
     int strips, rows, segs;     // in-plane walks: strips of columns, segments of `rows` rows
+    int cols;                   // FP64 tiles: columns of a tile (rows: its rows)
     int zstrips, zrows, zsegs;  // walks along z (3D split step)
     unsigned spin_limit;   // polls of a barrier wait before it gives up
     unsigned* err;         // DEV_ERR_TIMEOUT when a barrier wait ran out
