@@ -467,6 +467,7 @@ __global__ void __launch_bounds__(TX * TY, (TX * TY >= 256 ? 2 : 4))
     const int lx = tid % TX, ly = tid / TX;
     const FieldGeom& g = sg.f;
 
+    step_begin();
     if (tid == 0) {
         // dt from the max wave-speed sum of the input state, in FP64 once per
         // CTA (FP64 throughput is small on this part); every sweep of a split

@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(256, PairCfg<DIM, LAYOUT, SCHEME>::MIN_CTAS)
 
     // step scalars formed by thread 0 in FP64 and rounded to FP32 once
     float* sdt = reinterpret_cast<float*>(smem + 256);
+    step_begin();
     if (tid == 0) {
         // dt from the max wave-speed sum of the input state, in FP64 once per CTA
         const double dt = prm.cfl / __longlong_as_double((long long)ctl->smax[prm.slot_in]);

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(256, 2)
 
     // step scalars formed by thread 0 in FP64 and rounded to FP32 once
     float* sdt = reinterpret_cast<float*>(smem + 256);
+    step_begin();
     if (tid == 0) {
         const double dt = prm.cfl / __longlong_as_double((long long)ctl->smax[prm.slot_in]);
         sdt[0] = (float)dt;

@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(512, 1)
     const int lx = 2 * lane;  // this lane's cells of the row: lx, lx + 1
     const FieldGeom& g = sg.f;
 
+    step_begin();
     // step scalars formed by thread 0 in FP64 and rounded to FP32 once
     if (tid == 0) {
         const double dt = prm.cfl / __longlong_as_double((long long)ctl->smax[prm.slot_in]);

@@ -37,7 +37,7 @@ int tile64_occ()
 // measured times per step (4 us + 0.033 us per instruction): 64^2 with 8 x 4
 // tiles 7.4 us (modelled 7.4), 128^2 16 x 7 8.7 (9.1), 8 x 7 9.5 (9.7),
 // 256^2 16 x 14 19.7 (20), 512^2 16 x 27 63.8 (64), 1024^2 16 x 27 240 (244),
-// 32 x 17 258 (260), 16 x 7 270 (275).
+// 32 x 17 258 (260), 16 x 7 270 (294).
 void tile64_plan(WalkStep& a, int sms)
 {
     const int nx = a.g.n[0], ny = a.g.n[1];

@@ -67,9 +67,26 @@ struct SweepEntry {
                 if (e != cudaSuccess) return e;
                 configured = true;
             }
-            k<<<L.grid, C::NT, C::SMEM, L.stream>>>(*L.map_in, *L.map_out, static_cast<T*>(L.out), L.ctl, L.sg,
-                                                    L.prm);
-            return cudaGetLastError();
+            // Short steps are placed while the last CTAs of the one before run
+            // (step_begin): us a step, without / with, MUSCL-Hancock 20^3 11.7 / 9.5,
+            // 48^3 15.8 / 13.8, AoS 17.5 / 14.7, 64^3 21.7 / 19.6; Rusanov 96^3 37.1 /
+            // 35.9; FP64 2D MUSCL-Hancock 128^2 28.2 / 26.0, FORCE 34.4 / 28.8.  CTAs
+            // placed as others leave spread less evenly over the SMs, which costs more
+            // than the gap when a step is long or its CTAs take several items: 96^3
+            // MUSCL-Hancock (12 planes an item) 43.7 / 45.3, 256^3 517 / 539, AoS 626 /
+            // 651, FP64 2D MUSCL-Hancock 300^2 (380 items) 98.5 / 109.
+            const bool ahead = L.sg.items <= L.grid && L.sg.zchunk <= (SCHEME == SCHEME_MUSCL ? 8 : 16);
+            cudaLaunchAttribute dep{};
+            dep.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            dep.val.programmaticStreamSerializationAllowed = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(L.grid);
+            cfg.blockDim = dim3(C::NT);
+            cfg.dynamicSmemBytes = C::SMEM;
+            cfg.stream = L.stream;
+            cfg.attrs = &dep;
+            cfg.numAttrs = ahead ? 1 : 0;
+            return cudaLaunchKernelEx(&cfg, k, *L.map_in, *L.map_out, static_cast<T*>(L.out), L.ctl, L.sg, L.prm);
         }
     }
     static int smem() { return fits ? C::SMEM : 0; }

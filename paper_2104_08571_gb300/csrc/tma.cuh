@@ -268,4 +268,15 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// First statement of a step kernel that touches device memory comes after this:
+// a step launched as the programmatic dependent of the one before it may start
+// while that one's last CTAs run, and waits here until it has completed and its
+// stores are visible.  The step after this one may then start likewise, so at
+// most one launch is ahead.  (No effect in a launch without the attribute.)
+__device__ __forceinline__ void step_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 }  // namespace ripple
