@@ -16,15 +16,16 @@
 //   * four cells per thread stay in registers for the whole visit; neighbours
 //     in the warp come by shuffles, those in the thread from registers, and
 //     only the layers between two warps pass through shared memory;
-//   * kFimInner sweeps run between two exchanges of those layers, so a CTA
+//   * in FP32 two sweeps run between two exchanges of those layers, so a CTA
 //     barrier (which also decides convergence) is paid once per exchange;
 //   * everything a visit reads is requested at once: both buffers' values with
 //     the words that say which one counts, so the visit starts after one trip
 //     to L2 instead of three;
-//   * the update has no branches.
+//   * the FP32 update has no branches.
 // (Before: cells in shared memory, five loads and a barrier per sweep.)
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 #include "field.cuh"
 
@@ -59,7 +60,20 @@ __device__ __forceinline__ float fim_min3(float a, float b, float c)
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ double fim_min3(double a, double b, double c) { return fmin(fmin(a, b), c); }
+
+// Minimum of two values that are not negative (travel times and infinity): as
+// integers, off the FP64 pipe.
+__device__ __forceinline__ float fim_min(float a, float b) { return fmin(a, b); }
+__device__ __forceinline__ double fim_min(double a, double b)
+{
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return __longlong_as_double(x < y ? x : y);
+}
+__device__ __forceinline__ double fim_max(double a, double b)
+{
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return __longlong_as_double(x < y ? y : x);
+}
 
 // Godunov upwind local solver: a[d] = smaller neighbour value along axis d,
 // f = s * h.  Written for the distance u above the smallest neighbour, without
@@ -73,11 +87,33 @@ __device__ __forceinline__ double fim_min3(double a, double b, double c) { retur
 // Only differences enter the roots, so nothing of size T^2 cancels.  Infinite
 // neighbours give infinite or NaN distances, which the minimum or the
 // comparison passes over; f = inf gives inf (a cell that keeps its value).
+// FP64 branches instead: a warp whose cells are all one-sided skips the roots,
+// and FP64 issues at 1/64 of the FP32 rate (48 x 40 x 62: 3.6 ms a solve with
+// the branches, 4.1 without).
 template <typename T, int DIM>
 __device__ __forceinline__ T godunov(T a0, T a1, T a2, T f)
 {
     const T ff = f * f;
-    if (DIM == 2) {
+    if constexpr (std::is_same<T, double>::value) {
+        T x = fim_min(a0, a1), y = fim_max(a0, a1);
+        if (DIM == 2) {
+            const T d = a0 - a1;
+            if (!(fabs(d) < f)) return x + f;
+            return T(0.5) * (a0 + a1 + fim_sqrt(T(2) * f * f - d * d));
+        }
+        const T z = fim_max(y, a2), m = fim_min(y, a2);
+        y = fim_max(x, m);
+        x = fim_min(x, m);
+        T t = x + f;
+        if (!(t > y)) return t;
+        const T d = x - y;
+        t = T(0.5) * (x + y + fim_sqrt(T(2) * f * f - d * d));
+        if (!(t > z)) return t;
+        // 3 f^2 less the squared pairwise differences: no terms of size T^2 cancel
+        const T dxz = x - z, dyz = y - z;
+        const T disc = fmax(T(3) * f * f - (d * d + dxz * dxz + dyz * dyz), T(0));
+        return (x + y + z + fim_sqrt(disc)) * (T(1) / T(3));
+    } else if (DIM == 2) {
         const T lo = fmin(a0, a1), d = fmin(fmax(a0, a1) - lo, f);
         return lo + T(0.5) * (d + fim_sqrt(T(2) * ff - d * d));
     } else {
@@ -97,11 +133,17 @@ struct EikTile {
     static constexpr int CELLS = DIM == 2 ? TS * TS : TS * TS * TS;
     static constexpr int CPT = 4;           // cells per thread: rows (2D) or z layers (3D)
     static constexpr int NT = CELLS / CPT;  // threads per tile: 8 warps (2D), 4 warps (3D)
-    // a visit ends unconverged after this many: visits are cheapest when almost
-    // all of them converge (2048^2: 1509 us at 96, 1700 at 64, 2826 at 48)
-    static constexpr int MAX_SWEEPS = DIM == 2 ? 96 : 64;
 };
-constexpr int kFimInner = 2;  // sweeps between two exchanges (2048^2: 1 1674, 2 1509, 4 1540 us)
+// Sweeps between two exchanges (2048^2 FP32: 1 1674, 2 1509, 4 1540 us).  FP64
+// takes plain Jacobi sweeps: what the exchange costs is little beside a sweep's
+// FP64 work, and a second sweep on old layers is work that does not help.
+template <typename T>
+constexpr int kFimInner = sizeof(T) == 8 ? 1 : 2;
+// A visit ends unconverged after this many sweeps: visits are cheapest when
+// almost all of them converge (2048^2 FP32: 1509 us at 96, 1700 at 64, 2826 at
+// 48).  FP64: 64 and 48, six tile sides in 3D.
+template <typename T, int DIM>
+constexpr int kFimMaxSweeps = sizeof(T) == 8 ? (DIM == 2 ? 64 : 48) : (DIM == 2 ? 96 : 64);
 
 // Per-problem state of the FIM iteration.  Two bookkeeping schemes use it:
 //   flags (the batched runtime): act[3][ntiles] active flags and cur[2][ntiles]
@@ -192,12 +234,14 @@ struct FimSmem;
 template <typename T>
 struct FimSmem<T, 2> {
     T top[2][8][32], bot[2][8][32];  // first and last row of each warp
+    unsigned chg[2][8][4];           // lanes whose cell c changed, per warp (FP64)
     unsigned side_mask;
 };
 template <typename T>
 struct FimSmem<T, 3> {
     T zl[2][4][32];    // each warp's layer at the tile's middle in z
     T yl[2][4][4][8];  // each warp's rows at the tile's middle in y, [z][x]
+    unsigned chg[2][4][4];  // lanes whose cell c changed, per warp (FP64)
     unsigned side_mask;
 };
 
@@ -305,6 +349,13 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
     bool converged = false, moved = true;
     int sweeps = 0, par = 0;
     T lo = rg, hi = rg;  // the neighbours of the run's first and last cell
+    // FP64: the lanes whose cell c changed in the last sweep.  A cell none of
+    // whose neighbours changed keeps its value, and a warp skips a row or layer
+    // of such cells: FP64 arithmetic is what a sweep costs.
+    constexpr bool F64 = std::is_same<T, double>::value;
+    unsigned chg[CPT];
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) chg[c] = 0xffffffffu;
     for (;;) {
         // exchange the layers between warps; the barrier also tells whether any
         // cell has moved since the last one
@@ -322,11 +373,15 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
                 }
             }
         }
+        if (F64 && lane == 0) {
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) sm.chg[par][w][c] = chg[c];
+        }
         if (!__syncthreads_or(moved ? 1 : 0)) {
             converged = true;
             break;
         }
-        if (sweeps >= C::MAX_SWEEPS) break;
+        if (sweeps >= kFimMaxSweeps<T, DIM>) break;
         if constexpr (DIM == 2) {
             if (w > 0) lo = sm.bot[par][w - 1][lane];
             if (w < 7) hi = sm.top[par][w + 1][lane];
@@ -339,30 +394,85 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
             }
         }
         moved = false;
+        if constexpr (F64) {
+            // cells with a neighbour that changed (warp-uniform masks)
+            unsigned need[CPT];
 #pragma unroll
-        for (int s = 0; s < kFimInner; ++s) {
+            for (int c = 0; c < CPT; ++c) {
+                const unsigned m = chg[c];
+                if (DIM == 2) {
+                    need[c] = m << 1 | m >> 1;
+                } else {
+                    need[c] = (m << 1 & 0xfefefefeu) | (m >> 1 & 0x7f7f7f7fu) | m << 8 | m >> 8;
+                    const unsigned o = sm.chg[par][w ^ 1][c];
+                    need[c] |= (w & 1) == 0 ? o << 24 : o >> 24;
+                }
+                if (c > 0) need[c] |= chg[c == 0 ? 0 : c - 1];
+                if (c < CPT - 1) need[c] |= chg[c == CPT - 1 ? c : c + 1];
+            }
+            if (DIM == 2) {
+                if (w > 0) need[0] |= sm.chg[par][w - 1][CPT - 1];
+                if (w < 7) need[CPT - 1] |= sm.chg[par][w + 1][0];
+            } else if (r_lo) {
+                need[CPT - 1] |= sm.chg[par][w ^ 2][0];
+            } else {
+                need[0] |= sm.chg[par][w ^ 2][CPT - 1];
+            }
             T nv[CPT];
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
-                // at the warp's edges the shuffle returns the cell's own value, which
-                // changes nothing (a candidate above the cell's value is dropped),
-                // and the ghost is the third operand (infinite elsewhere)
-                const T l = __shfl_up_sync(0xffffffffu, v[c], 1, W), r = __shfl_down_sync(0xffffffffu, v[c], 1, W);
+                nv[c] = v[c];
+                chg[c] = 0u;
+                if (need[c] == 0u) continue;
+                T l = __shfl_up_sync(0xffffffffu, v[c], 1, W), r = __shfl_down_sync(0xffffffffu, v[c], 1, W);
+                if (xlo) l = xg[c];
+                if (xhi) r = xg[c];
                 const T below = c == 0 ? lo : v[c == 0 ? 0 : c - 1], above = c == CPT - 1 ? hi : v[c == CPT - 1 ? c : c + 1];
-                T g;
-                if constexpr (DIM == 2) {
-                    g = godunov<T, 2>(fim_min3(l, r, xg[c]), fmin(below, above), INF, f[c]);
-                } else {
+                const T ax = fim_min(l, r), ar = fim_min(below, above);
+                T ay = INF;
+                if (DIM == 3) {
                     const T u = __shfl_up_sync(0xffffffffu, v[c], 8), d = __shfl_down_sync(0xffffffffu, v[c], 8);
-                    g = godunov<T, 3>(fim_min3(l, r, xg[c]), fim_min3(u, d, yg[c]), fmin(below, above), f[c]);
+                    ay = fim_min(lane < 8 ? yg[c] : u, lane >= 24 ? yg[c] : d);
                 }
-                nv[c] = fmin(v[c], g);
-                moved |= v[c] - nv[c] >= tol;
+                bool down = false;
+                if (need[c] >> lane & 1u) {
+                    const T g = DIM == 2 ? godunov<T, 2>(ax, ar, INF, f[c]) : godunov<T, 3>(ax, ay, ar, f[c]);
+                    down = g < v[c];
+                    if (down) {
+                        moved |= v[c] - g >= tol;
+                        nv[c] = g;
+                    }
+                }
+                chg[c] = __ballot_sync(0xffffffffu, down);
             }
 #pragma unroll
             for (int c = 0; c < CPT; ++c) v[c] = nv[c];
+        } else {
+#pragma unroll
+            for (int s = 0; s < kFimInner<T>; ++s) {
+                T nv[CPT];
+#pragma unroll
+                for (int c = 0; c < CPT; ++c) {
+                    // at the warp's edges the shuffle returns the cell's own value, which
+                    // changes nothing (a candidate above the cell's value is dropped),
+                    // and the ghost is the third operand (infinite elsewhere)
+                    const T l = __shfl_up_sync(0xffffffffu, v[c], 1, W), r = __shfl_down_sync(0xffffffffu, v[c], 1, W);
+                    const T below = c == 0 ? lo : v[c == 0 ? 0 : c - 1], above = c == CPT - 1 ? hi : v[c == CPT - 1 ? c : c + 1];
+                    T g;
+                    if constexpr (DIM == 2) {
+                        g = godunov<T, 2>(fim_min3(l, r, xg[c]), fmin(below, above), INF, f[c]);
+                    } else {
+                        const T u = __shfl_up_sync(0xffffffffu, v[c], 8), d = __shfl_down_sync(0xffffffffu, v[c], 8);
+                        g = godunov<T, 3>(fim_min3(l, r, xg[c]), fim_min3(u, d, yg[c]), fmin(below, above), f[c]);
+                    }
+                    nv[c] = fmin(v[c], g);
+                    moved |= v[c] - nv[c] >= tol;
+                }
+#pragma unroll
+                for (int c = 0; c < CPT; ++c) v[c] = nv[c];
+            }
         }
-        sweeps += kFimInner;
+        sweeps += kFimInner<T>;
         par ^= 1;
     }
     updates += (long long)sweeps * C::CELLS;
