@@ -163,8 +163,9 @@ RIPPLE_API ripple_status ripple_field_describe(ripple_field field, ripple_field_
  *   0 = one cell per thread, 32 x 8 tiles; 1 = the same, 32 x 4 tiles;
  *   2 = packed cell pairs, 32 x 8 tiles (FP32); 3 = one warp per 64-cell row,
  *   64 x 14 tiles (FP32 3D MUSCL-Hancock only).
- * Automatic: FP32 2D fields and the FP32 split FORCE step run on strip walks
- * (several steps per launch, no variant number).
+ * Automatic: FP32 2D fields and the FP32 split FORCE step run on strip walks,
+ * FP64 2D first-order fields on tiles sized by the field (several steps per
+ * launch, no variant number).
  * zchunk: planes per z work item of 3D sweeps (0 = automatic: the chunk that
  * fills the resident blocks best).
  * RIPPLE_ERR_INVALID for an unknown variant or a negative zchunk; a variant
