@@ -75,56 +75,69 @@ __device__ __forceinline__ double fim_max(double a, double b)
     return __longlong_as_double(x < y ? y : x);
 }
 
-// Godunov upwind local solver: a[d] = smaller neighbour value along axis d,
-// f = s * h.  Written for the distance u above the smallest neighbour, without
-// branches:
-//   2D: u is the larger root of u^2 + (u - d)^2 = f^2, d the distance between
-//       the two; at d = f the root is f, the one-sided value, so clamping d at
-//       f covers both cases;
-//   3D (sorted, p and q the distances to the second and third): the 2D value
-//       of the first two, or, if that exceeds q, the larger root of u^2 + (u -
-//       p)^2 + (u - q)^2 = f^2.
-// Only differences enter the roots, so nothing of size T^2 cancels.  Infinite
-// neighbours give infinite or NaN distances, which the minimum or the
-// comparison passes over; f = inf gives inf (a cell that keeps its value).
-// FP64 branches instead: a warp whose cells are all one-sided skips the roots,
-// and FP64 issues at 1/64 of the FP32 rate (48 x 40 x 62: 3.6 ms a solve with
-// the branches, 4.1 without).
-template <typename T, int DIM>
-__device__ __forceinline__ T godunov(T a0, T a1, T a2, T f)
+// Godunov upwind local solver in FP64: a[d] = smaller neighbour value along
+// axis d, f = s * h.  It branches: a warp whose cells are all one-sided skips
+// the roots, and FP64 issues at 1/64 of the FP32 rate (48 x 40 x 62: 3.6 ms a
+// solve with the branches, 4.1 without).
+template <int DIM>
+__device__ __forceinline__ double godunov(double a0, double a1, double a2, double f)
 {
-    const T ff = f * f;
-    if constexpr (std::is_same<T, double>::value) {
-        T x = fim_min(a0, a1), y = fim_max(a0, a1);
-        if (DIM == 2) {
-            const T d = a0 - a1;
-            if (!(fabs(d) < f)) return x + f;
-            return T(0.5) * (a0 + a1 + fim_sqrt(T(2) * f * f - d * d));
-        }
-        const T z = fim_max(y, a2), m = fim_min(y, a2);
-        y = fim_max(x, m);
-        x = fim_min(x, m);
-        T t = x + f;
-        if (!(t > y)) return t;
-        const T d = x - y;
-        t = T(0.5) * (x + y + fim_sqrt(T(2) * f * f - d * d));
-        if (!(t > z)) return t;
-        // 3 f^2 less the squared pairwise differences: no terms of size T^2 cancel
-        const T dxz = x - z, dyz = y - z;
-        const T disc = fmax(T(3) * f * f - (d * d + dxz * dxz + dyz * dyz), T(0));
-        return (x + y + z + fim_sqrt(disc)) * (T(1) / T(3));
-    } else if (DIM == 2) {
-        const T lo = fmin(a0, a1), d = fmin(fmax(a0, a1) - lo, f);
-        return lo + T(0.5) * (d + fim_sqrt(T(2) * ff - d * d));
-    } else {
-        const T lo = fmin(a0, a1), hi = fmax(a0, a1);
-        const T x = fmin(lo, a2), z = fmax(hi, a2), y = fmax(lo, fmin(hi, a2));
-        const T p = y - x, q = z - x, d = fmin(p, f);
-        const T u2 = T(0.5) * (d + fim_sqrt(T(2) * ff - d * d));
-        const T disc = fmax(T(3) * ff - T(2) * (p * (p - q) + q * q), T(0));
-        const T u3 = (p + q + fim_sqrt(disc)) * (T(1) / T(3));
-        return x + (u2 > q ? u3 : u2);
+    double x = fim_min(a0, a1), y = fim_max(a0, a1);
+    if (DIM == 2) {
+        const double d = a0 - a1;
+        if (!(fabs(d) < f)) return x + f;
+        return 0.5 * (a0 + a1 + fim_sqrt(2.0 * f * f - d * d));
     }
+    const double z = fim_max(y, a2), m = fim_min(y, a2);
+    y = fim_max(x, m);
+    x = fim_min(x, m);
+    double t = x + f;
+    if (!(t > y)) return t;
+    const double d = x - y;
+    t = 0.5 * (x + y + fim_sqrt(2.0 * f * f - d * d));
+    if (!(t > z)) return t;
+    // 3 f^2 less the squared pairwise differences: no terms of size T^2 cancel
+    const double dxz = x - z, dyz = y - z;
+    const double disc = fmax(3.0 * f * f - (d * d + dxz * dxz + dyz * dyz), 0.0);
+    return (x + y + z + fim_sqrt(disc)) * (1.0 / 3.0);
+}
+
+// min(v, G) in FP32, G the Godunov value of a cell whose value is v; ff2 = 2 f^2.
+// Without branches: the candidates with one, two and three neighbours are all
+// formed, and each further one counts while the next neighbour lies below the
+// value so far (it is then the smaller one).
+//   one: the smallest neighbour x plus f, rounded once, at any scale of f.  The
+//       others square f and hold where f^2 is a normal number.
+//   two: x + u, u the larger root of u^2 + (u - p)^2 = f^2, p the distance from
+//       x to the second neighbour y;
+//   three: x + u, u the larger root of u^2 + (u - p)^2 + (u - q)^2 = f^2, q the
+//       distance from x to the third neighbour z.
+// Only differences enter the roots, so nothing of size T^2 cancels.  Comparing
+// with min(v, ...) passes over neighbours that are not below v, which could
+// only give a candidate above v: infinite ones (their candidates may be NaN),
+// and the cell's own value, which the shuffles return at a warp's edges.  f =
+// inf (a cell that keeps its value) gives v.
+// (A form with p clamped at f, so that the root covers one-sided cells too, is
+// as fast but rounds them through the root: f/2 where f^2 vanishes, below 1e-19,
+// and no value where it overflows, above 1e19.)
+template <int DIM>
+__device__ __forceinline__ float godunov_min(float a0, float a1, float a2, float f, float ff2, float v)
+{
+    const float lo = fmin(a0, a1), hi = fmax(a0, a1);
+    if (DIM == 2) {
+        const float p = hi - lo, two = fmaf(0.5f, p + fim_sqrt(fmaf(-p, p, ff2)), lo);
+        const float m = fmin(v, lo + f);
+        return hi < m ? fmin(m, two) : m;
+    }
+    const float x = fmin(lo, a2), z = fmax(hi, a2), y = fmax(lo, fmin(hi, a2));
+    const float p = y - x, q = z - x;
+    const float two = fmaf(0.5f, p + fim_sqrt(fmaf(-p, p, ff2)), x);
+    // 3 f^2 - 2 (p^2 - p q + q^2)
+    const float g = fmaf(p, q - p, -q * q), disc = fmaf(1.5f, ff2, g + g);
+    const float three = fmaf(1.f / 3.f, p + q + fim_sqrt(disc), x);
+    float m = fmin(v, x + f);
+    m = y < m ? fmin(m, two) : m;
+    return z < m ? fmin(m, three) : m;
 }
 
 template <int DIM>
@@ -354,8 +367,12 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
     // of such cells: FP64 arithmetic is what a sweep costs.
     constexpr bool F64 = std::is_same<T, double>::value;
     unsigned chg[CPT];
+    T ff2[CPT];  // 2 f^2 (FP32)
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) chg[c] = 0xffffffffu;
+    for (int c = 0; c < CPT; ++c) {
+        chg[c] = 0xffffffffu;
+        ff2[c] = T(2) * f[c] * f[c];
+    }
     for (;;) {
         // exchange the layers between warps; the barrier also tells whether any
         // cell has moved since the last one
@@ -436,7 +453,7 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
                 }
                 bool down = false;
                 if (need[c] >> lane & 1u) {
-                    const T g = DIM == 2 ? godunov<T, 2>(ax, ar, INF, f[c]) : godunov<T, 3>(ax, ay, ar, f[c]);
+                    const T g = DIM == 2 ? godunov<2>(ax, ar, INF, f[c]) : godunov<3>(ax, ay, ar, f[c]);
                     down = g < v[c];
                     if (down) {
                         moved |= v[c] - g >= tol;
@@ -453,19 +470,17 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
                 T nv[CPT];
 #pragma unroll
                 for (int c = 0; c < CPT; ++c) {
-                    // at the warp's edges the shuffle returns the cell's own value, which
-                    // changes nothing (a candidate above the cell's value is dropped),
-                    // and the ghost is the third operand (infinite elsewhere)
+                    // at the warp's edges the shuffle returns the cell's own value, which the
+                    // solver passes over, and the ghost is the third operand (infinite elsewhere)
                     const T l = __shfl_up_sync(0xffffffffu, v[c], 1, W), r = __shfl_down_sync(0xffffffffu, v[c], 1, W);
                     const T below = c == 0 ? lo : v[c == 0 ? 0 : c - 1], above = c == CPT - 1 ? hi : v[c == CPT - 1 ? c : c + 1];
-                    T g;
                     if constexpr (DIM == 2) {
-                        g = godunov<T, 2>(fim_min3(l, r, xg[c]), fmin(below, above), INF, f[c]);
+                        nv[c] = godunov_min<2>(fim_min3(l, r, xg[c]), fmin(below, above), INF, f[c], ff2[c], v[c]);
                     } else {
                         const T u = __shfl_up_sync(0xffffffffu, v[c], 8), d = __shfl_down_sync(0xffffffffu, v[c], 8);
-                        g = godunov<T, 3>(fim_min3(l, r, xg[c]), fim_min3(u, d, yg[c]), fmin(below, above), f[c]);
+                        nv[c] = godunov_min<3>(fim_min3(l, r, xg[c]), fim_min3(u, d, yg[c]), fmin(below, above), f[c],
+                                               ff2[c], v[c]);
                     }
-                    nv[c] = fmin(v[c], g);
                     moved |= v[c] - nv[c] >= tol;
                 }
 #pragma unroll
