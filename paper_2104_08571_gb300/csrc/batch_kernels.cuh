@@ -99,8 +99,9 @@ __device__ __forceinline__ T batch_wave_sum(const T (&q)[4], T gamma, T gm1, con
         const float p = __fmul_rn(gm1, __fmaf_rn(-0.5f, __fmul_rn(mm, inv), q[3]));
         ok = (q[0] > 0.f) & (p > 0.f);
         const float c = sqrt_v(__fmul_rn(__fmul_rn(gamma, p), inv));
-        const float s = __fmul_rn(__fadd_rn(fabsf(__fmul_rn(q[1], inv)), c), inv_dx[0]);
-        return __fmaf_rn(__fadd_rn(fabsf(__fmul_rn(q[2], inv)), c), inv_dx[1], s);
+        const float s0 = __fmul_rn(__fadd_rn(fabsf(__fmul_rn(q[1], inv)), c), inv_dx[0]);
+        const float s1 = __fmul_rn(__fadd_rn(fabsf(__fmul_rn(q[2], inv)), c), inv_dx[1]);
+        return __fadd_rn(s0, s1);
     } else {
         return wave_sum<T, 2>(q, gamma, gm1, inv_dx, ok);
     }

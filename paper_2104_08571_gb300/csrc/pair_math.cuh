@@ -149,10 +149,10 @@ __device__ __forceinline__ void pflux_y(const f2 (&q)[4], f2 inv_rho, f2 p, f2 (
 }
 
 // Wave-speed sums sum_d (|u_d| + c)/dx_d of a pair of conserved states and
-// their admissibility (density and pressure > 0) per lane.  The sum is written
-// with fused multiply-adds: left as products and sums, the compiler was seen to
-// fuse them all the same, and the scalar form of the batched step has to agree
-// bit for bit.
+// their admissibility (density and pressure > 0) per lane.  Products and sums
+// are separate roundings, so the sum does not depend on which of two axes comes
+// first.  The additions are scalar: a packed product and sum get contracted
+// into a fused multiply-add in spite of .rn (seen in every kernel that used them).
 template <int DIM>
 __device__ __forceinline__ f2 wave_sum2(const f2 (&q)[DIM + 2], f2 gamma, f2 gm1, const f2 (&inv_dx)[3], bool& ok0,
                                         bool& ok1)
@@ -167,7 +167,10 @@ __device__ __forceinline__ f2 wave_sum2(const f2 (&q)[DIM + 2], f2 gamma, f2 gm1
     const f2 c = sqrt_v(gamma * p * inv_rho);
     f2 s = (abs_v(q[1] * inv_rho) + c) * inv_dx[0];
 #pragma unroll
-    for (int d = 1; d < DIM; ++d) s = fma_v(abs_v(q[1 + d] * inv_rho) + c, inv_dx[d], s);
+    for (int d = 1; d < DIM; ++d) {
+        const f2 t = (abs_v(q[1 + d] * inv_rho) + c) * inv_dx[d];
+        s = f2{__fadd_rn(s.x, t.x), __fadd_rn(s.y, t.y)};
+    }
     return s;
 }
 
