@@ -34,6 +34,7 @@
 
 #include "fim_tile.cuh"
 #include "grid_sync.cuh"
+#include "resident.h"
 #include "runtime.h"
 
 namespace ripple {
@@ -268,11 +269,8 @@ ripple_status fim_solve_lists(FimProblem<T> a, void* scratch, FieldCtl* ctl, lon
     e.spin_limit = grid_spin_limit();
     e.ctl = ctl;
     auto kern = fim_kernel<T, DIM>;
-    static const int resident = [&] {  // CTAs per SM, 0 on error
-        int c = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, EikTile<DIM>::NT, 0) == cudaSuccess ? c : 0;
-    }();
-    int per_sm = resident;
+    static ResidentCtas resident;
+    int per_sm = resident.get(kern, EikTile<DIM>::NT, 0);
     if (per_sm < 1) return fail(RIPPLE_ERR_INTERNAL, "FIM kernel cannot be resident");
     // 2D solves keep 100 to 300 tiles active per iteration, and an iteration
     // lasts as long as its longest visit: two CTAs per SM give most visits

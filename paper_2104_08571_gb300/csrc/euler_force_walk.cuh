@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_force_walk_kernel(co
 
 }  // namespace ripple
 
+#include "resident.h"
 #include "runtime.h"
 
 namespace ripple {
@@ -297,15 +298,8 @@ namespace ripple {
 template <int DIM, int LAYOUT>
 static int force_walk_occupancy()  // resident CTAs per SM, 0 if the kernel cannot run
 {
-    static const int n = [] {
-        auto kern = euler_force_walk_kernel<DIM, LAYOUT>;
-        int c = 0;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, force_smem<DIM>()) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, kWalkWarps * 32, force_smem<DIM>()) != cudaSuccess)
-            return 0;
-        return c;
-    }();
-    return n;
+    static ResidentCtas resident;
+    return resident.get(euler_force_walk_kernel<DIM, LAYOUT>, kWalkWarps * 32, force_smem<DIM>());
 }
 template <int DIM, int LAYOUT>
 static cudaError_t force_walk_run(const WalkStep& a, int grid, cudaStream_t s)

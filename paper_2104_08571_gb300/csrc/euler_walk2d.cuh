@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_walk2d_kernel(const 
 
 }  // namespace ripple
 
+#include "resident.h"
 #include "runtime.h"
 
 namespace ripple {
@@ -284,16 +285,8 @@ namespace ripple {
 template <int SCHEME, int LAYOUT>
 static int walk2d_occupancy()
 {
-    static const int n = [] {
-        auto kern = euler_walk2d_kernel<SCHEME, LAYOUT>;
-        int c = 0;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Walk2D<SCHEME>::SMEM) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, kWalkWarps * 32, Walk2D<SCHEME>::SMEM) != cudaSuccess)
-            return 0;
-        return c;
-    }();
-    return n;
+    static ResidentCtas resident;
+    return resident.get(euler_walk2d_kernel<SCHEME, LAYOUT>, kWalkWarps * 32, Walk2D<SCHEME>::SMEM);
 }
 template <int SCHEME, int LAYOUT>
 static cudaError_t walk2d_run(const WalkStep& a, int grid, cudaStream_t s)

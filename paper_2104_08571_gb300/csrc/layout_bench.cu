@@ -17,6 +17,7 @@
 // through registers on its way in or out.
 #include <cstdint>
 
+#include "resident.h"
 #include "runtime.h"
 #include "tma.cuh"
 
@@ -246,12 +247,10 @@ RIPPLE_API ripple_status ripple_particle_update(ripple_ctx ctx, int64_t n, float
     const bool soa = layout == RIPPLE_SOA;
     const bool aligned = ap % 16 == 0 && (soa ? n % 4 == 0 : n % 2 == 0);
     if (staged && aligned) {
-        static bool configured[2] = {false, false};
+        static ResidentCtas resident[2];
         auto k = soa ? particle_staged_kernel<LAYOUT_SOA> : particle_staged_kernel<LAYOUT_AOS>;
-        if (!configured[soa ? 1 : 0]) {
-            RIPPLE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kStagedSmem));
-            configured[soa ? 1 : 0] = true;
-        }
+        if (resident[soa ? 1 : 0].get(k, 256, kStagedSmem) == 0)  // also opts in to the shared memory
+            return fail(RIPPLE_ERR_CUDA, "the staged particle kernel does not fit on this device");
         const long long nchunks = (n + 2047) / 2048;
         const int grid = (int)std::min<long long>(nchunks, 2LL * ctx->sm_count);
         k<<<grid, 256, kStagedSmem, ctx->stream>>>(n, dt, particles);

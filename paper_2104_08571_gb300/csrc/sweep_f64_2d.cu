@@ -18,16 +18,8 @@ cudaError_t tile64_launch(const WalkStep& a, int grid, cudaStream_t s)
 }
 int tile64_occ()
 {
-    static const int n = [] {
-        int c = 0;
-        if (cudaFuncSetAttribute(euler_tile64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTile64Smem) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, euler_tile64_kernel, kTile64Threads, kTile64Smem) !=
-                cudaSuccess)
-            return 0;
-        return c;
-    }();
-    return n;
+    static ResidentCtas resident;
+    return resident.get(euler_tile64_kernel, kTile64Threads, kTile64Smem);
 }
 // Sides of a tile: the ones that give the fullest SM the fewest FP64
 // instructions per scheduler (counts per lane of the three lists of

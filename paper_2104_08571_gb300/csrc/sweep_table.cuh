@@ -6,6 +6,7 @@
 #include "euler_sweep_pair.cuh"
 #include "euler_sweep_pair3.cuh"
 #include "euler_sweep_row3.cuh"
+#include "resident.h"
 #include "runtime.h"
 
 namespace ripple {
@@ -61,12 +62,7 @@ struct SweepEntry {
             return cudaErrorInvalidValue;
         } else {
             auto k = K::fn();
-            static bool configured = false;
-            if (!configured) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-                if (e != cudaSuccess) return e;
-                configured = true;
-            }
+            if (occupancy() == 0) return cudaErrorInvalidValue;  // also opts in to the shared memory
             // Short steps are placed while the last CTAs of the one before run
             // (step_begin): us a step, without / with, MUSCL-Hancock 20^3 11.7 / 9.5,
             // 48^3 15.8 / 13.8, AoS 17.5 / 14.7, 64^3 21.7 / 19.6; Rusanov 96^3 37.1 /
@@ -95,15 +91,8 @@ struct SweepEntry {
         if constexpr (!fits) {
             return 0;
         } else {
-            static const int n = [] {  // the same on every device the library is built for
-                auto k = K::fn();
-                int c = 0;
-                if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess ||
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k, C::NT, C::SMEM) != cudaSuccess)
-                    return 0;
-                return c;
-            }();
-            return n;
+            static ResidentCtas resident;
+            return resident.get(K::fn(), C::NT, C::SMEM);
         }
     }
 };
