@@ -735,7 +735,9 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
         return best;
     };
     int v = U->variant, zc = U->zchunk;
-    if (v < 0 || sweep_smem(U->dtype, U->ndim, layout, scheme, v) == 0) {
+    // the chosen variant, if it exists for this dtype, dimension and scheme
+    const bool chosen = v >= 0 && sweep_smem(U->dtype, U->ndim, layout, scheme, v) > 0;
+    if (!chosen) {
         // default: the packed pair kernel (FP32), else the first that fits
         v = sweep_smem(U->dtype, U->ndim, layout, scheme, kPairVariant) > 0 ? kPairVariant : -1;
         for (int c = 0; c < kNumSweepVariants && v < 0; ++c)
@@ -812,7 +814,7 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     // (per step, tiles of euler_sweep.cuh -> now: 64^2 17.5 -> 7.4 us, 256^2
     // 36 -> 19.7 us, 1024^2 380 -> 240 us)
     const bool walks = U->dtype == RIPPLE_F32 ? U->ndim == 2 || split : U->ndim == 2 && scheme == SCHEME_RUSANOV1;
-    if (walks && U->variant < 0) {
+    if (walks && !chosen) {
         st = walk_field_steps(U, *p, scheme, layout, nsteps);
         if (st != RIPPLE_OK) return st;
         nsteps_left = 0;
