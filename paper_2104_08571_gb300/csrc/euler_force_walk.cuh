@@ -281,10 +281,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_force_walk_kernel(co
         walk_reduce(ctl, (rs + 1) % 3, smax, red);
         if (s + 1 < a.K && !grid_barrier(&ctl->bar[0], ++phase, a.spin_limit, sflag)) break;
     }
-    if (sflag[0]) {
-        if (tid == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
-        return;
-    }
+    if (sflag[0] && tid == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
     walk_leave(ctl);
 }
 

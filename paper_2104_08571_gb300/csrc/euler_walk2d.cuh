@@ -268,10 +268,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) euler_walk2d_kernel(const 
         walk_reduce(ctl, (rs + 1) % 3, smax, red);
         if (s + 1 < a.K && !grid_barrier(&ctl->bar[0], (unsigned)(s + 1), a.spin_limit, sflag)) break;
     }
-    if (sflag[0]) {
-        if (tid == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
-        return;
-    }
+    if (sflag[0] && tid == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
     walk_leave(ctl);
 }
 

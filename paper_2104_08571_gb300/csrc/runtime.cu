@@ -279,10 +279,7 @@ ripple_status take_device_error(ripple_field f)
     RIPPLE_CUDA(cudaMemcpyAsync(&h->err, &f->ctl->err, sizeof(unsigned), cudaMemcpyDeviceToHost, f->ctx->stream));
     RIPPLE_CUDA(cudaStreamSynchronize(f->ctx->stream));
     const unsigned err = h->err;
-    if (err) {
-        RIPPLE_CUDA(cudaMemsetAsync(&f->ctl->err, 0, sizeof(unsigned), f->ctx->stream));
-        RIPPLE_CUDA(cudaMemsetAsync(f->ctl->bar, 0, sizeof(f->ctl->bar) + sizeof(f->ctl->work), f->ctx->stream));
-    }
+    if (err) RIPPLE_CUDA(cudaMemsetAsync(&f->ctl->err, 0, sizeof(unsigned), f->ctx->stream));
     return map_dev_err(err);
 }
 
@@ -864,7 +861,6 @@ ripple_status ripple_fv_step(ripple_field U, const ripple_fv_params* p, int64_t 
     if (host.err) {
         RIPPLE_CUDA(cudaMemsetAsync(&U->ctl->err, 0, sizeof(unsigned), s));
         RIPPLE_CUDA(cudaMemsetAsync(&U->ctl->counters[4], 0, 4 * sizeof(long long), s));
-        RIPPLE_CUDA(cudaMemsetAsync(U->ctl->bar, 0, sizeof(U->ctl->bar) + sizeof(U->ctl->work), s));  // after a wait that ran out
         return map_dev_err(host.err, &host);
     }
     return RIPPLE_OK;

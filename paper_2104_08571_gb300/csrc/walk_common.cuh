@@ -47,7 +47,10 @@ struct WalkStep {
 // lines, which a second CTA on the SM would still be working on: 230 against
 // 169 us a step for 4096^2 FORCE with two CTAs of 8 warps per SM.  One CTA of
 // 16 has no such neighbour.)
-// Every CTA calls this once, after its last barrier.
+// Every CTA calls this once, after its last barrier; one whose wait ran out too:
+// it arrives at no further barrier, so the others' waits run out as well and
+// the last of them leaves the words at zero for whatever is queued behind this
+// launch before the host has seen the error.
 __device__ __forceinline__ void walk_leave(FieldCtl* ctl)
 {
     __syncthreads();
