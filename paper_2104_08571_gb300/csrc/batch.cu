@@ -26,6 +26,7 @@
 #include "euler_solo2d.cuh"
 #include "grid_sync.cuh"
 #include "runtime.h"
+#include "step_budget.h"
 
 namespace ripple {
 
@@ -1076,7 +1077,6 @@ static void collect_finished(BatchRuntime* rt)
 //     its iterations were scheduled, so the bits are the same).
 // Requests arriving meanwhile are admitted after the round.  More resident
 // problems than that run in batched rounds, where one launch steps all of them.
-constexpr long long kSoloMaxSteps = 1024;
 // FP64 Euler problems of at least this many cells (512^2) run alone when they
 // are the oldest; smaller ones, and FP32 ones of any size, gain from sharing a
 // batched launch (FP32 walks: a 1000^2 step takes 11 us alone and 13 us in a
@@ -1088,10 +1088,6 @@ static long long solo_big_cells(ripple_dtype dt) { return dt == RIPPLE_F64 ? 1LL
 // chain per step (64^2 3.4 against 4.0, 256^2 4.1 / 4.6, 512^2 6.9 / 6.0, 1024^2
 // 15.4 / 11.2 us a step)
 constexpr long long kSoloWalkCells = 160000;
-
-// Solo GPU seconds an FP32 Euler step of `cells` cells takes (a fit of the
-// multi-step solvers on GB300: a fixed barrier and dt cost, then the cells).
-static double solo_step_seconds(double cells) { return 3.5e-6 + 7.5e-12 * cells; }
 
 static ripple_status solo_round(BatchRuntime* rt, bool& handled)
 {
@@ -1147,10 +1143,7 @@ static ripple_status solo_round(BatchRuntime* rt, bool& handled)
         handled = true;
         const ripple_request& r = in->req;
         const long long cells = r.dims[0] * r.dims[1];
-        // a launch of about a millisecond at most, so arrivals wait little
-        const double est_step = solo_step_seconds((double)cells);
-        const long long K = std::min<long long>(
-            r.nsteps - in->steps_done, std::max<long long>(8, std::min<long long>(kSoloMaxSteps, (long long)(1e-3 / est_step))));
+        const long long K = solo_steps(dt == RIPPLE_F64, cells, r.nsteps - in->steps_done);
         RIPPLE_CUDA(cudaEventRecord(rt->ev_r0, s));
         if (dt == RIPPLE_F32 && cells >= kSoloWalkCells) {
             // the single-field walks on the instance's buffers and control block

@@ -10,6 +10,7 @@
 
 #include "grid_sync.cuh"
 #include "runtime.h"
+#include "step_budget.h"
 
 namespace ripple {
 
@@ -329,14 +330,6 @@ static void walk_split(long long lines, int n, int sms, double extra, int most, 
     }
 }
 
-// Steps of a walk launch: about 64 M cell updates, so that a launch stays near
-// a millisecond (a long call is then cut into several launches).
-static int walk_steps(const FieldGeom& g, int64_t left)
-{
-    const long long cells = (long long)g.n[0] * g.n[1] * g.n[2];
-    return (int)std::min<long long>(left, std::max(1LL, std::min(256LL, (64LL << 20) / cells)));
-}
-
 // Geometry, parameters and work split of a walk launch; returns its grid.
 static int walk_plan(const ripple_ctx_s* ctx, WalkStep& a, const FieldGeom& g, bool f64, int scheme, double gamma,
                      double cfl, const double* dx, int bc, int occ)
@@ -362,7 +355,7 @@ static int walk_plan(const ripple_ctx_s* ctx, WalkStep& a, const FieldGeom& g, b
     a.strips = (g.n[0] + kWalkUse - 1) / kWalkUse;
     walk_split((long long)a.strips * g.n[2], g.n[1], sms, scheme == SCHEME_RUSANOV1 ? 1.5 : 2.0, d3 ? 24 : 128, &a.rows,
                &a.segs);
-    // unit numbers are 32-bit: at most 2^32 padded cells and at least 60 cells per unit row
+    // unit numbers are 32-bit: at most 2^32 padded cells, and a row (at least 8 of them) gives a unit per 60 columns
     long long units = (long long)a.strips * a.segs * g.n[2];
     if (d3) {
         a.zstrips = (g.n[0] + 63) / 64;
@@ -660,7 +653,7 @@ static ripple_status walk_field_steps(ripple_field U, const ripple_fv_params& p,
     a.err = &U->ctl->err;
     const int grid = walk_plan(ctx, a, g, f64, scheme, p.gamma, p.cfl, p.dx, (int)p.bc, occ);
     for (int64_t done = 0; done < nsteps;) {
-        a.K = walk_steps(g, nsteps - done);
+        a.K = walk_steps(f64, (long long)g.n[0] * g.n[1] * g.n[2], nsteps - done);
         a.cur = U->cur;
         a.slot = (int)(U->steps_total % 3);
         a.first = done == 0;
