@@ -592,7 +592,7 @@ def bench_batched(R, torch, local, nsteps=100, count=512, keep=None):
         "speedup_vs_loop": t_loop / t_batch,
         "max_rel_l1_vs_loop": worst,
         "autotune": {"layout": "SoA" if cfg["layout"] == R.RIPPLE_SOA else "AoS",
-                     "tile": ["32x8", "8x32", "16x16"][cfg["tile_variant"]],
+                     "tile": "none" if cfg["staging"] == 2 else ["32x8", "8x32", "16x16"][cfg["tile_variant"]],
                      "staging": ["tma", "direct", "walk"][cfg["staging"]],
                      "ms_per_global_step": {
                          f"{['tma', 'direct', 'walk'][k[2]]}/{'SoA' if k[0] == R.RIPPLE_SOA else 'AoS'}/"

@@ -359,12 +359,17 @@ RIPPLE_API ripple_status ripple_wait(ripple_ctx ctx, uint64_t ticket, int64_t ti
 RIPPLE_API ripple_status ripple_batch_get_stats(ripple_ctx ctx, ripple_batch_stats* out);
 
 /*
- * Autotuner: time the batched step for each halo staging (TMA, direct, walk),
- * layout (SoA, AoS) and tile shape on n sample Euler problems of the given
- * square sides (dtype `dtype`), and return the fastest in *chosen (other fields
- * of *chosen are kept).  ms_per_step (nullable) receives 3 x 2 x 3 timings (the
- * walk staging has no tile shape: its three entries per layout are equal),
- * index (staging * 2 + layout_index) * 3 + tile_variant, SoA = layout index 0.
+ * Autotuner: time the batched step, launched step by step, for each halo
+ * staging (TMA, direct, walk), layout (SoA, AoS) and tile shape on n sample
+ * Euler problems of the given square sides (dtype `dtype`), and return the
+ * fastest in *chosen (other fields of *chosen are kept).  ms_per_step (nullable)
+ * receives 3 x 2 x 3 timings, index (staging * 2 + layout_index) * 3 +
+ * tile_variant, SoA = layout index 0.  The walk staging has no tile shape: its
+ * three entries per layout are equal, and tile_variant 0 is returned with it.
+ * FP32 steps of staging 0 are the walks of staging 2: its entries are copies of
+ * those, and 2 is returned.  Dependency-driven rounds are not timed: they take
+ * walk units with the staging 2 that is returned, tiles of shape tile_variant
+ * with 0 or 1.
  * Does not change the context's configuration (pass *chosen to
  * ripple_batch_configure).
  */

@@ -1571,10 +1571,10 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
     ripple_status status = RIPPLE_OK;
     for (int sg = 0; sg < kNumBatchStagings && status == RIPPLE_OK; ++sg)
     for (int li = 0; li < 2 && status == RIPPLE_OK; ++li) {
+        if (step_staging(dt, sg) != sg) continue;  // its steps are another staging's, timed there
         const ripple_layout lay = li == 0 ? RIPPLE_SOA : RIPPLE_AOS;
         for (int v = 0; v < kNumBatchVariants && status == RIPPLE_OK; ++v) {
-            const int run = step_staging(dt, sg);  // what a step of that staging runs
-            const bool walk = run == kBatchStagingWalk;  // walk units: the tile shape does not apply
+            const bool walk = sg == kBatchStagingWalk;  // walk units: the tile shape does not apply
             if (walk && v > 0) {
                 if (ms) ms[(sg * 2 + li) * kNumBatchVariants + v] = ms[(sg * 2 + li) * kNumBatchVariants];
                 continue;
@@ -1683,13 +1683,13 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
                 break;
             }
             const int lay_i = lay == RIPPLE_SOA ? LAYOUT_SOA : LAYOUT_AOS;
-            const int grid = std::max(1, batch_occupancy(dt, lay_i, v, run)) * ctx->sm_count;
+            const int grid = std::max(1, batch_occupancy(dt, lay_i, v, sg)) * ctx->sm_count;
             for (int k = 0; k < 3 && ce == cudaSuccess; ++k)
-                ce = launch_batch_step(dt, lay_i, v, run, grid, s, d_e, nullptr, d_t, d_c, 0);
+                ce = launch_batch_step(dt, lay_i, v, sg, grid, s, d_e, nullptr, d_t, d_c, 0);
             cudaEventRecord(e0, s);
             const int reps = 6;
             for (int k = 0; k < reps && ce == cudaSuccess; ++k)
-                ce = launch_batch_step(dt, lay_i, v, run, grid, s, d_e, nullptr, d_t, d_c, 0);
+                ce = launch_batch_step(dt, lay_i, v, sg, grid, s, d_e, nullptr, d_t, d_c, 0);
             cudaEventRecord(e1, s);
             cudaStreamSynchronize(s);
             float el = 0.f;
@@ -1710,6 +1710,11 @@ static ripple_status autotune(ripple_ctx ctx, const int64_t* sides, int n, rippl
                 best->staging = sg;
             }
         }
+    }
+    for (int sg = 0; sg < kNumBatchStagings && ms && status == RIPPLE_OK; ++sg) {
+        const int run = step_staging(dt, sg);
+        for (int i = 0; i < 2 * kNumBatchVariants && run != sg; ++i)
+            ms[sg * 2 * kNumBatchVariants + i] = ms[run * 2 * kNumBatchVariants + i];
     }
     cudaStreamDestroy(s);
     return status;
