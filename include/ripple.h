@@ -227,7 +227,8 @@ typedef struct {
 typedef struct {
     int64_t iterations;  /* active-list iterations run */
     int64_t tile_visits; /* tile relaxations performed */
-    int64_t cell_updates;/* Godunov cell updates performed (tile visits x sweeps x cells) */
+    int64_t cell_updates;/* Godunov cell updates performed: tile visits x sweeps x cells, in FP64 without
+                            the cells that a sweep passes over because no neighbour has changed */
 } ripple_eik_stats;
 
 /*

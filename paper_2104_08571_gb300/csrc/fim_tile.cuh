@@ -248,14 +248,14 @@ template <typename T>
 struct FimSmem<T, 2> {
     T top[2][8][32], bot[2][8][32];  // first and last row of each warp
     unsigned chg[2][8][4];           // lanes whose cell c changed, per warp (FP64)
-    unsigned side_mask;
+    unsigned side_mask, done;
 };
 template <typename T>
 struct FimSmem<T, 3> {
     T zl[2][4][32];    // each warp's layer at the tile's middle in z
     T yl[2][4][4][8];  // each warp's rows at the tile's middle in y, [z][x]
     unsigned chg[2][4][4];  // lanes whose cell c changed, per warp (FP64)
-    unsigned side_mask;
+    unsigned side_mask, done;
 };
 
 // Visit tile t of problem `a` in iteration k (all threads of the CTA call it)
@@ -367,6 +367,7 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
     // of such cells: FP64 arithmetic is what a sweep costs.
     constexpr bool F64 = std::is_same<T, double>::value;
     unsigned chg[CPT];
+    unsigned done = 0;  // cells this warp has updated (FP64)
     T ff2[CPT];  // 2 f^2 (FP32)
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
@@ -441,6 +442,7 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
                 nv[c] = v[c];
                 chg[c] = 0u;
                 if (need[c] == 0u) continue;
+                done += __popc(need[c]);
                 T l = __shfl_up_sync(0xffffffffu, v[c], 1, W), r = __shfl_down_sync(0xffffffffu, v[c], 1, W);
                 if (xlo) l = xg[c];
                 if (xhi) r = xg[c];
@@ -490,11 +492,10 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
         sweeps += kFimInner<T>;
         par ^= 1;
     }
-    updates += (long long)sweeps * C::CELLS;
-
     // ---- write back; boundary-layer changes activate neighbours ----
-    if (tid == 0) sm.side_mask = 0u;
+    if (tid == 0) sm.side_mask = sm.done = 0u;
     __syncthreads();
+    if (F64 && lane == 0) atomicAdd(&sm.done, done);
     T* out = a.buf[1 - cb];
     bool any = false, first = false, last = false;
 #pragma unroll
@@ -533,6 +534,7 @@ __device__ __forceinline__ void fim_visit_tile(FimSmem<T, DIM>& sm, const FimPro
         }
         if (nb >= 0) book.activate(nb);
     }
+    updates += F64 ? (long long)sm.done : (long long)sweeps * C::CELLS;
     __syncthreads();
 }
 
