@@ -43,7 +43,7 @@ BYTES_PER_CELL_UPDATE = 40  # FP32, 5 components: 20 B read + 20 B written per c
 # DRAM bytes per cell update of the sweep kernel (the row kernel, SoA) as measured by ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum of one 256x256x128 launch, divided by its cells);
 # traffic scales with the cells of a launch.  Re-measure whenever the kernel changes.
-DRAM_BYTES_PER_CELL_UPDATE = (216594688 + 137211392) / (256 * 256 * 128)
+DRAM_BYTES_PER_CELL_UPDATE = (220964864 + 137028608) / (256 * 256 * 128)
 METRIC = "cell-updates/s"
 ACTIVE_CELLS = 4 << 20  # serving: per-step cell budget of stepped Euler problems
 
@@ -122,7 +122,7 @@ class ClockSampler:
 # capture of each solve (smsp__inst_executed.sum x 32 / the solve's Godunov
 # updates); the eikonal roofline is issue-bound, so these set its achieved
 # rate.  Re-measure whenever the kernels change.
-FIM_INSTR_PER_UPDATE = {"2d_2048": 38.44, "3d_192": 85.87}
+FIM_INSTR_PER_UPDATE = {"2d_2048": 26.08, "3d_192": 57.25}
 
 
 def eikonal_roofline(name, updates_per_s, clocks, sms):
@@ -405,8 +405,8 @@ def bench_solo(R, torch, local, sides=(64, 256, 1024), nsteps=400):
     """One 2D Euler request (sine density, FP32, periodic Rusanov, 400 steps)
     served alone, per side: on the multi-step solo solver (solo rounds), on the
     batched step launched once per step (solo rounds off; the results must be
-    the same bits), and through the single-field API's per-step launch loop
-    on a device-resident field."""
+    the same bits), and through one call of the single-field API (its
+    multi-step kernels) on a device-resident field."""
     out = {}
     ctx = R.ripple_ctx_create(local)
     clk = ClockSampler(local).__enter__()
@@ -602,9 +602,9 @@ def bench_batched(R, torch, local, nsteps=100, count=512, keep=None):
 
 def bench_force_split(R, torch, local, par=None, legs=None):
     """The paper's own Euler solver (dimensionally split sweeps, x then y [then
-    z], FORCE face flux), one sweep launch per axis: 2D FP32 8192^2 periodic sine
-    density (a Table flux size), 3D FP32 256^3 blast (the headline state,
-    transmissive), and the 2D FP64 128^2 workload."""
+    z], FORCE face flux): 2D FP32 8192^2 periodic sine density (a Table flux
+    size), 3D FP32 256^3 blast (the headline state, transmissive), and the 2D
+    FP64 128^2 workload (one sweep launch per axis; FP32 sweeps are fused)."""
     ctx = R.ripple_ctx_create(local)
     R.use_torch_allocator(ctx, local)
     stream = torch.cuda.Stream(device=local)

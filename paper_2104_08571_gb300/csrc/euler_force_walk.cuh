@@ -35,8 +35,8 @@
 // no registers and no wait involves another thread.
 //
 // Measured (SoA, per step, one sweep per launch before -> now): 4096^2 250 ->
-// 117 us, 256^3 630 -> 302 us, 200 x 171 x 186 300 -> 135 us, 64^3 19 us.
-// Bound by issue: 163 thread instructions per cell update in 2D at 61 % issue;
+// 117 us, 256^3 630 -> 290 us, 200 x 171 x 186 300 -> 135 us, 64^3 19 us.
+// Bound by issue: 164 thread instructions per cell update in 2D at 62 % issue;
 // HBM would allow 80 us at 4096^2.
 #pragma once
 #include "walk_common.cuh"

@@ -251,8 +251,8 @@ __device__ __forceinline__ void muscl_states(const T (&qm)[DIM + 2], const T (&q
 }
 
 // Separately rounded product and sum (never contracted into a fused
-// multiply-add): the wave-speed sum then does not depend on the order of the
-// axes, so a problem and its axis-permuted twin get the same dt.
+// multiply-add): the wave-speed sum then does not depend on which of the first
+// two axes comes first.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
